@@ -261,6 +261,10 @@ struct lms_batch_plan {
         Cand *best = nullptr;           // device
     } cls[3];
     int *hvec = nullptr;                // device, per set
+    // sets of the one-kernel branch-and-bound (direct.cu), largest first
+    int ndirect = 0, direct_teams = 0, direct_nmax = 0;
+    int *direct_sets = nullptr;         // device
+    void *direct_mem = nullptr;
     // sweep sets
     std::vector<long long> off_host;
     std::vector<int> sweep_sets;        // global indices, assigned to streams
@@ -312,13 +316,24 @@ int lms_batch_plan_create_ex(const int64_t *offsets_host, int64_t B, const int32
         p->hval[i] = h;
     }
     // classes
-    std::vector<int> members[3];
+    std::vector<int> members[3], direct;
     for (int64_t i = 0; i < B; ++i) {
         const int64_t n = offsets_host[i + 1] - offsets_host[i];
         if (n <= p->plain_max) members[n <= 64 ? 0 : (n <= 128 ? 1 : 2)].push_back((int)i);
+        else if (n <= DIRECT_BATCH_MAX && direct_ok((int)n, p->hval[i])) direct.push_back((int)i);
         else p->sweep_sets.push_back((int)i);
     }
-    size_t bytes = a256(sizeof(int) * B);
+    std::sort(direct.begin(), direct.end(), [&](int a, int b) {
+        return offsets_host[a + 1] - offsets_host[a] > offsets_host[b + 1] - offsets_host[b];
+    });
+    if (!direct.empty()) {
+        p->ndirect = (int)direct.size();
+        p->direct_nmax = (int)(offsets_host[direct[0] + 1] - offsets_host[direct[0]]);
+        p->direct_teams = direct_batch_teams(p->ndirect, p->direct_nmax, sms);
+        if (p->direct_teams < 1) { delete p; return LMS_ERR_CUDA; }
+    }
+    size_t bytes = a256(sizeof(int) * B) + a256(sizeof(int) * direct.size()) +
+                   (p->ndirect ? direct_batch_bytes(p->direct_teams, p->direct_nmax) : 0);
     std::vector<std::vector<long long>> pres(3);
     for (int c = 0; c < 3; ++c) {
         p->cls[c].E = 2 << c;
@@ -340,6 +355,11 @@ int lms_batch_plan_create_ex(const int64_t *offsets_host, int64_t B, const int32
     auto take = [&](size_t b) { void *r = q; q += a256(b); return r; };
     p->hvec = (int *)take(sizeof(int) * B);
     cudaMemcpy(p->hvec, p->hval.data(), sizeof(int) * B, cudaMemcpyHostToDevice);
+    if (p->ndirect) {
+        p->direct_sets = (int *)take(sizeof(int) * direct.size());
+        cudaMemcpy(p->direct_sets, direct.data(), sizeof(int) * direct.size(), cudaMemcpyHostToDevice);
+        p->direct_mem = take(direct_batch_bytes(p->direct_teams, p->direct_nmax));
+    }
     for (int c = 0; c < 3; ++c) {
         auto &C = p->cls[c];
         C.sets = (int *)take(sizeof(int) * members[c].size());
@@ -419,7 +439,11 @@ int lms_fit_batched(lms_batch_plan *p, const void *xv, const void *yv, const int
         cudaEventRecord(p->ev_start, st);
         for (int s = 0; s < p->nstreams; ++s) cudaStreamWaitEvent(p->streams[s], p->ev_start, 0);
     }
-    // plain classes on the caller's stream
+    // direct sets, then the plain classes, on the caller's stream
+    bool failed = false;
+    if (p->ndirect)
+        failed = launch_direct_batch(x, y, off, p->hvec, p->direct_sets, p->ndirect, p->direct_nmax, p->direct_teams,
+                                     p->plain_max, p->bnb_min, out, p->direct_mem, st) != cudaSuccess;
     for (int c = 0; c < 3; ++c) {
         auto &C = p->cls[c];
         if (C.nsets == 0) continue;
@@ -447,7 +471,6 @@ int lms_fit_batched(lms_batch_plan *p, const void *xv, const void *yv, const int
     // sweep sets on their streams
     int sms = 1;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    bool failed = false;
     for (size_t k = 0; k < p->sweep_sets.size() && !failed; ++k) {
         const int i = p->sweep_sets[k];
         const int s = p->stream_of[k];

@@ -12,6 +12,7 @@ enum Stage {
     STAGE_PACK, STAGE_SAMPLE, STAGE_SAMPLE_SORT, STAGE_SPLITTERS, STAGE_COUNT_PAIRS, STAGE_PREFIX,
     STAGE_SCAN, STAGE_SCATTER, STAGE_SEGSORT, STAGE_SEGSORT_BIG, STAGE_PLAN, STAGE_INIT, STAGE_SWEEP,
     STAGE_ARGMIN, STAGE_PLAIN, STAGE_OTHER, STAGE_NODE_LB, STAGE_SEEDS, STAGE_SETNET, STAGE_HOUGH, STAGE_TREE,
+    STAGE_DIRECT,
     STAGE_COUNT
 };
 
@@ -192,6 +193,24 @@ unsigned long long workspace_generation();
 // captured graph, added to the launch counter
 bool profiling_on();
 void add_launches(long long count);
+
+// ---------------------------------------------------------------- one-kernel branch and bound (direct.cu)
+// whether a fit of n points with order statistic h takes it (a small h leaves
+// too many intervals alive, see direct.cu)
+bool direct_ok(int n, int h);
+size_t direct_bytes(int n);   // device scratch of one fit
+// One fit by one thread-block cluster; the record reports `algo`.  pred: a
+// predicted slope on the device, or null.
+cudaError_t launch_direct(const short *x, const short *y, int n, int h, int algo, const float *pred, lms_result *out,
+                          void *mem, cudaStream_t st);
+// Many sets of at most nmax <= DIRECT_BATCH_MAX points, one CTA each: sets
+// (device) lists the set indices in the order they are handed out.
+constexpr int DIRECT_BATCH_MAX = 4096;
+int direct_batch_teams(int nsets, int nmax, int sms);   // resident CTAs, 0 on failure
+size_t direct_batch_bytes(int nteams, int nmax);
+cudaError_t launch_direct_batch(const short *x, const short *y, const long long *off, const int *hvec, const int *sets,
+                                int nsets, int nmax, int nteams, int plain_max, int bnb_min, lms_result *out,
+                                void *mem, cudaStream_t st);
 
 // ---------------------------------------------------------------- argmin
 cudaError_t launch_argmin(const Cand *cands, int count, lms_result *out, int algorithm, const int *err,
