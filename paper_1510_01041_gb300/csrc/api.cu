@@ -81,6 +81,7 @@ struct Choice {
     SweepPlan sweep;
     int plain_warps;
     int sms;
+    bool direct;      // by the one-kernel branch-and-bound (direct.cu)
     size_t bytes;
     size_t bnb_off;   // offset of the branch-and-bound scratch
     size_t f32_off;   // offset of the float32 sweep scratch
@@ -109,6 +110,7 @@ int choose(int n, int h, int dtype, const lms_options *opt, int dev, Choice &c)
     c.sms = sms;
     c.bnb_off = 0;
     c.f32_off = 0;
+    c.direct = algo_req == LMS_ALGO_AUTO && algo == LMS_ALGO_SWEEP && dtype == LMS_I16 && direct_ok(n, h);
     if (algo == LMS_ALGO_PLAIN) {
         if (n > 1024) return LMS_ERR_UNSUPPORTED;
         c.plain_warps = plain_warps_for(n, sms);
@@ -158,6 +160,11 @@ int run_fit(const void *x, const void *y, int n, int h, int dtype, const lms_opt
             cudaStream_t st, void *ws_in, const Choice &c)
 {
     cudaGetLastError();
+    if (c.direct)
+        return launch_direct((const short *)x, (const short *)y, n, h, LMS_ALGO_SWEEP, nullptr, out, ws_in, st) ==
+                       cudaSuccess
+                   ? LMS_OK
+                   : LMS_ERR_CUDA;
     if (c.algo == LMS_ALGO_PLAIN) {
         Cand *cands = static_cast<Cand *>(ws_in);
         if (launch_plain((const short *)x, (const short *)y, n, h, cands, c.plain_warps, st) != cudaSuccess)
@@ -216,10 +223,22 @@ int fit_bnb_after(const void *x, const void *y, int64_t n, int64_t h, const floa
     if (rc) return rc;
     int dev;
     if (current_device(dev)) return LMS_ERR_CUDA;
+    void *ws = nullptr;
+    // the statistics, the seed modes and the sweep's tuning options belong to
+    // the staged branch-and-bound; without them one kernel does it all
+    if (!stats && o.seed_mode == 0 && o.sweepers == 0 && o.buckets == 0 && direct_ok((int)n, (int)h)) {
+        rc = workspace(direct_bytes((int)n), st, &ws);
+        if (rc) return rc;
+        if (pred_ready && cudaStreamWaitEvent(st, pred_ready, 0) != cudaSuccess) return LMS_ERR_CUDA;
+        cudaGetLastError();
+        return launch_direct((const short *)x, (const short *)y, (int)n, (int)h, LMS_ALGO_BNB, seed_slope, out, ws,
+                             st) == cudaSuccess
+                   ? LMS_OK
+                   : LMS_ERR_CUDA;
+    }
     Choice c;
     rc = choose((int)n, (int)h, LMS_I16, &o, dev, c);
     if (rc) return rc;
-    void *ws = nullptr;
     rc = workspace(c.bytes, st, &ws);
     if (rc) return rc;
     SweepPlan p = c.sweep;
