@@ -21,6 +21,7 @@ namespace lms {
 namespace {
 
 constexpr int CHUNK = 64;   // slopes per work item of the plain kernel
+constexpr int BATCH_DIRECT_MIN = 65;    // sets from this size take one CTA of the one-kernel branch-and-bound
 constexpr int BATCH_BNB_MIN_N = 512;   // default size from which a set takes the branch-and-bound
 
 template <typename K>
@@ -319,7 +320,7 @@ int lms_batch_plan_create_ex(const int64_t *offsets_host, int64_t B, const int32
     std::vector<int> members[3], direct;
     for (int64_t i = 0; i < B; ++i) {
         const int64_t n = offsets_host[i + 1] - offsets_host[i];
-        if (n <= p->plain_max) members[n <= 64 ? 0 : (n <= 128 ? 1 : 2)].push_back((int)i);
+        if (n <= p->plain_max && (n < BATCH_DIRECT_MIN || !direct_ok((int)n, p->hval[i]))) members[n <= 64 ? 0 : (n <= 128 ? 1 : 2)].push_back((int)i);
         else if (n <= DIRECT_BATCH_MAX && direct_ok((int)n, p->hval[i])) direct.push_back((int)i);
         else p->sweep_sets.push_back((int)i);
     }

@@ -855,7 +855,9 @@ __host__ __device__ constexpr size_t pairs_bytes(int NC, int n)
 }
 
 // A superset of the distinct slopes of the pairs with key in [A, B), appended
-// to the team's list by one CTA.  wk: pairs_bytes(NC, n).  Narrow leaves hold
+// to the team's list by one CTA, which takes share `part` of `parts` of the
+// pairs or fractions (CTAs sharing a leaf may list a slope twice, which only
+// tests it twice).  wk: pairs_bytes(NC, n).  Narrow leaves hold
 // few reduced fractions p / q with q <= X at all (about 0.31 X^2 times the
 // width), far fewer than pairs when many pairs share a slope: up to
 // FRACTIONS of them the CTA tries every q.  p / q lies in the leaf when
@@ -865,7 +867,8 @@ __host__ __device__ constexpr size_t pairs_bytes(int NC, int n)
 template <int T>
 __device__ __noinline__ void list_pairs(const int *pts, int n, long long A, long long B, const Box &bx, int NC,
                                         unsigned char *wk, int *s_warp, const TeamMem &m,
-                                        int *nlist, int *over, int HC)
+                                        int *nlist, int *over, int HC,
+                                        int part, int parts)
 {
     const int xr = bx.xhi - bx.xlo, yr = bx.yhi - bx.ylo;
     if (fractions(A, B, xr) < FRACTIONS) {
@@ -873,7 +876,7 @@ __device__ __noinline__ void list_pairs(const int *pts, int n, long long A, long
         // |p| <= y range
         const long long nearest = A > 0 ? A : B < 0 ? -B : 0;
         const int qmax = nearest ? (int)min((long long)xr, (((long long)yr + 1) << 32) / nearest + 1) : xr;
-        for (int q = 1 + (int)threadIdx.x; q <= qmax; q += T) {
+        for (int q = 1 + part * T + (int)threadIdx.x; q <= qmax; q += T * parts) {
             const long long end = d * q;
             for (long long g = (unsigned)(0u - (unsigned)A * (unsigned)q); g < end; g += 1LL << 32) {
                 const int y = (int)((A * q + g) >> 32);
@@ -933,7 +936,7 @@ __device__ __noinline__ void list_pairs(const int *pts, int n, long long A, long
         // then the next cell) end to end and tests 32 of them at once.
         constexpr int L = T >= 32 ? 32 : 1;
         const int lane = threadIdx.x % L;
-        for (int e0 = threadIdx.x - lane; e0 < n; e0 += T) {
+        for (int e0 = part * T + threadIdx.x - lane; e0 < n; e0 += T * parts) {
             const int e = e0 + lane;
             int pa = 0, n1 = 0, nn = 0, beg2 = 0;
             if (e < n) {
@@ -970,13 +973,15 @@ __device__ __noinline__ void list_pairs(const int *pts, int n, long long A, long
                 const int b = ord[u < k1 ? e0 + src + 1 + u : k2 + u - k1];
                 int dy, dx;
                 if (!pair_slope(p, pts[b], dy, dx)) continue;
+                const long long t = (long long)dy << 32;
+                if (!steep && (A * dx > t || B * dx <= t)) continue;
                 const long long k = slope_key(dy, dx);
                 if (k >= A && k < B) table_put(tab, k, dx);
             }
         }
     }
     __syncthreads();
-    // append the table (leaves are disjoint: no other CTA lists these keys)
+    // append the table
     const int held = *tab.count;
     __shared__ int s_at;
     if (threadIdx.x == 0) {
@@ -1663,9 +1668,12 @@ __global__ void __launch_bounds__(T) k_direct(const DirectArgs A)
                 // ------------------------------------------------ distinct slopes of the leaves
                 int NC = T;
                 while (NC < n && NC < CELLS_MAX) NC <<= 1;
-                for (int l = rank; l < lfn; l += C)
-                    list_pairs<T>(pts, n, S.leaf[lf0 + l].a, S.leaf[lf0 + l].b, bx, NC, wk, S.warp_a, m,
-                                  &st->nlist[lpar], &st->over[lpar], sh.HC);
+                const int parts = max(1, (int)C / lfn);
+                for (int l = rank; l < lfn * parts; l += C) {
+                    const DNode &lf = S.leaf[lf0 + l / parts];
+                    list_pairs<T>(pts, n, lf.a, lf.b, bx, NC, wk, S.warp_a, m, &st->nlist[lpar], &st->over[lpar], sh.HC,
+                                  l % parts, parts);
+                }
                 team_sync();
                 const bool over = __ldcg(&st->over[lpar]) != 0;
                 const int nn = __ldcg(&st->nlist[lpar]);
@@ -1678,7 +1686,7 @@ __global__ void __launch_bounds__(T) k_direct(const DirectArgs A)
                         for (int k = threadIdx.x; k < nn; k += T) {
                             const long long v = s[k];
                             int r = 0;
-                            for (int j = 0; j < nn; ++j) r += s[j] < v;
+                            for (int j = 0; j < nn; ++j) r += s[j] < v || (s[j] == v && j < k);
                             m.ev[r] = v;
                             m.evd[r] = __ldcg(&m.lden[k]);
                         }
@@ -1695,7 +1703,8 @@ __global__ void __launch_bounds__(T) k_direct(const DirectArgs A)
                                 const int q = (lo + hi) >> 1;
                                 if (s[q] < v) lo = q + 1; else hi = q;
                             }
-                            m.evd[lo] = __ldcg(&m.lden[k]);
+                            const unsigned den = __ldcg(&m.lden[k]);
+                            for (; lo < nn && s[lo] == v; ++lo) m.evd[lo] = den;
                         }
                     }
                 }
@@ -1715,18 +1724,18 @@ __global__ void __launch_bounds__(T) k_direct(const DirectArgs A)
                         S.t1 = known ? t1 : 0;
                     }
                     __syncthreads();
-                    const int parts = min(nn, min(PM, max(8, NG)));
-                    for (int q = threadIdx.x; q < parts; q += T) {
+                    const int runs = min(nn, min(PM, max(8, NG)));
+                    for (int q = threadIdx.x; q < runs; q += T) {
                         DNode nd;
-                        nd.a = (long long)nn * q / parts;
-                        nd.b = (long long)nn * (q + 1) / parts;
+                        nd.a = (long long)nn * q / runs;
+                        nd.b = (long long)nn * (q + 1) / runs;
                         nd.t0 = S.t0;
                         nd.t1 = S.t1;
                         nd.est = 0.0f;
                         nd.force = 0;
                         S.work[cur][q] = nd;
                     }
-                    P = parts;
+                    P = runs;
                     lf0 += lfn;
                     if (lf0 == nleaf) {
                         lf0 = nleaf = 0;
