@@ -137,7 +137,11 @@ int choose(int n, int h, int dtype, const lms_options *opt, int dev, Choice &c)
     } else {
         return LMS_ERR_ARG;
     }
-    c.bytes += 256;   // result staging for host-pointer calls
+    c.bytes += 256;   // result staging for host-pointer calls, and the flag of a float fit
+    if (dtype == LMS_F32 && algo_req == LMS_ALGO_AUTO && direct_f32_ok(n, h) && direct_f32_bytes(n) + 256 <= c.bytes) {
+        c.direct = true;
+        c.direct_bytes = c.bytes;
+    }
     return LMS_OK;
 }
 
@@ -164,7 +168,7 @@ int run_fit(const void *x, const void *y, int n, int h, int dtype, const lms_opt
             cudaStream_t st, void *ws_in, const Choice &c)
 {
     cudaGetLastError();
-    if (c.direct)
+    if (c.direct && dtype == LMS_I16)
         return launch_direct((const short *)x, (const short *)y, n, h, c.algo, nullptr, out, ws_in, st) ==
                        cudaSuccess
                    ? LMS_OK
@@ -187,6 +191,15 @@ int run_fit(const void *x, const void *y, int n, int h, int dtype, const lms_opt
     }
     SweepPlan p = c.sweep;
     sweep_plan_carve(p, ws_in);
+    if (dtype == LMS_F32 && c.direct) {
+        // the one-kernel branch-and-bound first, on the same workspace; the
+        // sweep's kernels return at once when it has written the record
+        int *done = reinterpret_cast<int *>(static_cast<unsigned char *>(ws_in) + c.bytes - 64);
+        if (launch_direct_f32((const float *)x, (const float *)y, n, h, LMS_ALGO_SWEEP, out, done, ws_in, st) !=
+            cudaSuccess)
+            return LMS_ERR_CUDA;
+        p.skip = done;
+    }
     if (dtype == LMS_F32)
         return launch_sweep_f32_fit(p, (const float *)x, (const float *)y,
                                     static_cast<unsigned char *>(ws_in) + c.f32_off, out, st) == cudaSuccess

@@ -56,6 +56,9 @@ namespace {
 
 constexpr long long D_MAX = 0x7fffffffffffffffLL;
 constexpr long long D_GUARD = 1LL << 46;   // slope keys beyond it are used in units of 2^-26 (no overflow)
+constexpr int F_YS = 29;                   // float sets: units of 2^-29 of a grid step, slope keys of 2^-29
+constexpr int F_BITS = 29;                 // .. grid coordinates below 2^F_BITS
+constexpr long long F_KMAX = 1LL << 32;    // .. and slopes (of the scaled axes) below 8: projections below 2^62
 constexpr int STEEP = 6;                   // .. that is, without their last bits
 constexpr int NODE_F = 4;                  // children of an interval
 constexpr int EV_F = 8;                    // children of a run of slopes
@@ -65,6 +68,8 @@ constexpr float FRACTIONS = 1000.0f;         // expected fractions of a leaf up 
 constexpr int CELLS_MAX = 8192;             // cells of the pair search
 constexpr int WIDE_ITEMS = 2;              // up to so many questions a CTA, the whole CTA works on each
 constexpr int DEPTH_MAX = 28;              // levels: an interval has fewer than 2^48 keys, NODE_F^24
+constexpr int F_SCORES = 4096;             // slopes of a float set that are scored, else the sweep takes over
+constexpr int F_PHASES = 400;
 constexpr int PHASES_MAX = 1 << 20;        // phases of one fit before it is reported as failed
 constexpr int EV_DEPTH = 6;                // levels of a run of at most EV_F^EV_DEPTH slopes
 
@@ -89,6 +94,13 @@ struct TeamState {
 struct Answer {
     long long t0, t1;
     int keep, pad;
+};
+
+// Best float candidate: lexicographic (w, theta1, theta2, pair).
+struct CandD {
+    double w, s, t;
+    unsigned pair;
+    int valid;
 };
 
 // Sizes of one team's memory; the same on the host and the device.
@@ -125,7 +137,7 @@ __host__ __device__ inline long long team_bytes(const TeamShape &s)
     return d_up(sizeof(TeamState)) + d_up(sizeof(DNode) * (long long)stack_cap(s)) +
            d_up(sizeof(DNode) * (long long)estack_cap(s)) + d_up(2 * sizeof(Answer) * (long long)s.PM) +
            2 * d_up(8LL * s.HC) +
-           2 * d_up(4LL * s.HC) + d_up(sizeof(Cand) * (long long)s.PM) + d_up(4LL * s.ptsn) +
+           2 * d_up(4LL * s.HC) + d_up(sizeof(CandD) * (long long)s.PM) + d_up(4LL * s.ptsn) +
            d_up(s.sortw) * s.C;
 }
 
@@ -141,7 +153,7 @@ __device__ inline TeamMem team_carve(unsigned char *p, const TeamShape &s)
     m.lden = reinterpret_cast<unsigned *>(take(4LL * s.HC));
     m.ev = reinterpret_cast<long long *>(take(8LL * s.HC));
     m.evd = reinterpret_cast<unsigned *>(take(4LL * s.HC));
-    m.xres = reinterpret_cast<Cand *>(take(sizeof(Cand) * (long long)s.PM));
+    m.xres = reinterpret_cast<Cand *>(take(sizeof(CandD) * (long long)s.PM));   // or CandD
     m.pts = reinterpret_cast<int *>(take(4LL * s.ptsn));
     m.sort = p;
     return m;
@@ -310,8 +322,19 @@ __device__ __forceinline__ int slot_of(int b)
     return (b & ~31) | ((b ^ (b >> 5)) & 31);
 }
 
+// Float points are quantised to a grid of 2^30 steps a side (int2, see
+// k_direct); every other set is packed in 16-bit halves.
+using ::lms::px;
+using ::lms::py;
+__device__ __forceinline__ int px(int2 p) { return p.x; }
+__device__ __forceinline__ int py(int2 p) { return p.y; }
+
+__device__ __forceinline__ int packed_of(int p) { return p; }
+__device__ __forceinline__ int packed_of(int2) { return 0; }
+
 // z at slope K 2^-ys, in units of 2^-ys.
-__device__ __forceinline__ long long z_at(int p, long long K, int ys)
+template <class P>
+__device__ __forceinline__ long long z_at(P p, long long K, int ys)
 {
     return ((long long)py(p) << ys) - (long long)px(p) * K;
 }
@@ -362,8 +385,8 @@ __device__ __forceinline__ void hist_zero(const Group<G> &g, int *hist)
 // roundings in all, so |error| < NB 2^-20 = eps, which widens every interval.
 // Later passes are exact in 64-bit integers; they only look at [T0, T1], the
 // hull of the bins that reached depth h.
-template <int G, int NB>
-__device__ __noinline__ bool may_hold_at(const Group<G> &g, const int *pts, int n, int h, long long A, long long B,
+template <int G, int NB, class P>
+__device__ __noinline__ bool may_hold_at(const Group<G> &g, const P *pts, int n, int h, long long A, long long B,
                                          long long U, long long tol, const Box &bx, int *hist, long long &T0,
                                          long long &T1, int ys)
 {
@@ -411,7 +434,7 @@ __device__ __noinline__ bool may_hold_at(const Group<G> &g, const int *pts, int 
             hist_zero<G, NB>(g, hist);
 #pragma unroll 4
             for (int k = g.lane; k < n; k += G) {
-                const int p = pts[k];
+                const P p = pts[k];
                 const float x = (float)px(p), y = (float)py(p);
                 const float base = fmaf(y, sc, c0);
                 const float pa = fmaf(-x, fa, base), pb = fmaf(-x, fb, base);
@@ -439,7 +462,10 @@ __device__ __noinline__ bool may_hold_at(const Group<G> &g, const int *pts, int 
         // positions of interest lie within reach = (T1 - T0) + U + X (B - A)
         // + 2 of T0, so each of the five roundings is below 2^-24 reach.
         const long long reach = (T1 - T0) + U + (long long)(bx.xhi - bx.xlo) * (B - A) + (1LL << 33);
+        bool packed = false;
+        if constexpr (sizeof(P) == 4) {
         if (B - A < (1LL << 40) && reach < (1LL << 46) && (reach >> sh) < NB * 64) {
+            packed = true;
             const unsigned ta = (unsigned)(T0 >> 17), ah = (unsigned)(A >> 17), bh = (unsigned)(B >> 17);
             const float sc = pow2f(17 - sh), dn = pow2f(-sh);
             const float al = (float)(int)(A & 0x1ffff) * dn, bl = (float)(int)(B & 0x1ffff) * dn;
@@ -449,7 +475,7 @@ __device__ __noinline__ bool may_hold_at(const Group<G> &g, const int *pts, int 
             const float last = (float)(int)((T1 - T0) >> sh);
 #pragma unroll 4
             for (int k = g.lane; k < n; k += G) {
-                const int p = pts[k];
+                const int p = packed_of(pts[k]);
                 const int xi = px(p);
                 const unsigned yb = (unsigned)((int)(p & 0xffff0000) >> (33 - ys)) - ta;
                 const float xf = -(float)xi;
@@ -460,10 +486,12 @@ __device__ __noinline__ bool may_hold_at(const Group<G> &g, const int *pts, int 
                 atomicAdd(&hist[slot_of<NB / G>(round_int(fminf(fmaxf(s, 0.0f), last)))], 1);
                 atomicAdd(&hist[slot_of<NB / G>(round_int(fminf(fmaxf(e, 0.0f), last)) + 1)], -1);
             }
-        } else
+        }
+        }
+        if (!packed)
 #pragma unroll 2
         for (int k = g.lane; k < n; k += G) {
-            const int p = pts[k];
+            const P p = pts[k];
             const long long u = z_at(p, A, ys), v = z_at(p, B, ys);
             const long long s = min(u, v) - U, e = max(u, v);
             if (e < T0 || s > T1) continue;
@@ -482,11 +510,12 @@ __device__ __noinline__ bool may_hold_at(const Group<G> &g, const int *pts, int 
     return true;
 }
 
-template <int G, int NB>
-__device__ bool may_hold(const Group<G> &g, const int *pts, int n, int h, long long A, long long B, long long U,
+template <int G, int NB, class P>
+__device__ bool may_hold(const Group<G> &g, const P *pts, int n, int h, long long A, long long B, long long U,
                                       long long tol, const Box &bx, int *hist, long long &T0, long long &T1)
 {
     if (U < 0) return false;
+    if constexpr (sizeof(P) == 8) return may_hold_at<G, NB>(g, pts, n, h, A, B, U, tol, bx, hist, T0, T1, F_YS);
     int ys = 32;
     if (A <= -D_GUARD || B >= D_GUARD) {
         ys = 32 - STEEP;
@@ -598,13 +627,13 @@ __device__ __forceinline__ void hist_cumulate(const Group<G> &g, int *hist)
 // window that beats cur must start, when known.  The same two kinds of pass
 // as may_hold: float bins of the whole range (with `coarse` only that pass), then integer bins of
 // the regions where the narrowest windows start and end.
-template <int G, int NB>
-__device__ __noinline__ long long ub_at(const Group<G> &g, const int *pts, int n, int h, long long K, long long cur,
+template <int G, int NB, class P>
+__device__ __noinline__ long long ub_at(const Group<G> &g, const P *pts, int n, int h, long long K, long long cur,
                                         const Box &bx, int *hist, long long T0, long long T1,
                                         bool coarse = false)
 {
     const bool steep = K <= -D_GUARD || K >= D_GUARD;
-    const int ys = steep ? 32 - STEEP : 32;
+    const int ys = sizeof(P) == 8 ? F_YS : steep ? 32 - STEEP : 32;
     if (steep) {
         K >>= STEEP;   // some slope beside it
         cur = (cur >> STEEP) + 1;
@@ -633,7 +662,7 @@ __device__ __noinline__ long long ub_at(const Group<G> &g, const int *pts, int n
         hist_zero<G, NB>(g, hist);
 #pragma unroll 4
         for (int k = g.lane; k < n; k += G) {
-            const int p = pts[k];
+            const P p = pts[k];
             const float f = fmaf(-(float)px(p), fk, fmaf((float)py(p), sc, c0));
             atomicAdd(&hist[slot_of<NB / G>(round_int(fminf(fmaxf(f, 0.0f), (float)(NB - 1))))], 1);
         }
@@ -675,7 +704,10 @@ __device__ __noinline__ long long ub_at(const Group<G> &g, const int *pts, int n
         int q = 17;
         while (q < 24 && (reach >> (q + 30)) != 0) ++q;
         const long long span = hi2 - lo1 + (1LL << (q + 16));
+        bool packed = false;
+        if constexpr (sizeof(P) == 4) {
         if ((reach >> (q + 30)) == 0 && (span >> sh) < (1 << 18) && sh >= 4) {
+            packed = true;
             const unsigned tl = (unsigned)(lo1 >> q), kh = (unsigned)(K >> q);
             const float sc = pow2f(q - sh), dn = pow2f(-sh);
             const int low = (1 << q) - 1;
@@ -687,7 +719,7 @@ __device__ __noinline__ long long ub_at(const Group<G> &g, const int *pts, int n
             slack = 1LL << (sh - 2);
 #pragma unroll 4
             for (int k = g.lane; k < n; k += G) {
-                const int p = pts[k];
+                const int p = packed_of(pts[k]);
                 const int xi = px(p);
                 const unsigned d = ((unsigned)((int)(p & 0xffff0000) >> 16) << (ys - q)) - tl - (unsigned)xi * kh;
                 const float f = fmaf(-(float)xi, kl, fmaf((float)(int)d, sc, c0));
@@ -697,7 +729,9 @@ __device__ __noinline__ long long ub_at(const Group<G> &g, const int *pts, int n
                 else if (f < beg2 - 0.5f) ++mid;
                 else atomicAdd(&hist[slot_of<NB / G>(NB / 2 + round_int(fminf(fmaxf(f - beg2, 0.0f), (float)(NB / 2 - 1))))], 1);
             }
-        } else
+        }
+        }
+        if (!packed)
 #pragma unroll 2
         for (int k = g.lane; k < n; k += G) {
             const long long z = z_at(pts[k], K, ys);
@@ -746,6 +780,14 @@ __device__ __forceinline__ bool steep_above(long long A, long long B, int dh, in
     else if (A >= 0 && A < D_MAX) K = A;
     else return false;
     const __int128 v = (__int128)K * dh - ((__int128)yr << 32);
+    return v > (__int128)U;
+}
+
+// The same for every slope beyond F_KMAX of a float set (dh less one step, yr
+// more one step: the grid).
+__device__ __forceinline__ bool steep_above_at(long long K, int dh, int yr, long long U)
+{
+    const __int128 v = (__int128)K * (dh - 1) - ((__int128)(yr + 1) << F_YS);
     return v > (__int128)U;
 }
 
@@ -1006,6 +1048,216 @@ __device__ __noinline__ void list_pairs(const int *pts, int n, long long A, long
     __syncthreads();
 }
 
+// ------------------------------------------------------------------ float points
+struct FloatSet {
+    const float *x, *y;
+    double xc, yc, sx, sy;   // grid = rint((v - c) * s), s a power of two
+    double ratio;            // scaled slope = slope * ratio
+};
+
+__device__ __forceinline__ long long order_of(double v)
+{
+    const long long b = v == 0.0 ? 0LL : __double_as_longlong(v);
+    return b < 0 ? (b ^ 0x7fffffffffffffffLL) : b;
+}
+__device__ __forceinline__ double of_order(long long k)
+{
+    return __longlong_as_double(k < 0 ? (k ^ 0x7fffffffffffffffLL) : k);
+}
+__device__ __forceinline__ bool slope_f32(const FloatSet &f, int i, int j, double &s)
+{
+    double dx = (double)f.x[j] - (double)f.x[i], dy = (double)f.y[j] - (double)f.y[i];
+    if (dx == 0.0) return false;
+    if (dx < 0.0) { dx = -dx; dy = -dy; }
+    s = __ddiv_rn(dy, dx);
+    return true;
+}
+__device__ __forceinline__ double z_f32(const FloatSet &f, int k, double s)
+{
+    return __dsub_rn((double)f.y[k], __dmul_rn(s, (double)f.x[k]));
+}
+
+// The pairs whose slope lies in the leaf [A, B) of scaled slope keys, listed
+// by one CTA's share: slope bits and index pair.  Cells of z(A) as in
+// list_pairs; both points of a pair may lie half a step off the grid in x and
+// y, which widens the cells by (1 + |s|) steps.
+template <int T>
+__device__ __noinline__ void list_pairs_f32(const int2 *pts, int n, long long A, long long B, const Box &bx,
+                                            const FloatSet &f, int NC, unsigned char *wk, int *s_warp,
+                                            const TeamMem &m, int *nlist, int *over, int HC, int part, int parts)
+{
+    unsigned *cnt = reinterpret_cast<unsigned *>(wk);
+    unsigned short *ord = reinterpret_cast<unsigned short *>(cnt + NC);
+    for (int q = threadIdx.x; q < NC; q += T) cnt[q] = 0u;
+    __syncthreads();
+    const long long ka = max(A < 0 ? -A : A, B < 0 ? -B : B);
+    const unsigned long long width = (unsigned long long)(bx.xhi - bx.xlo) * (unsigned long long)(B - A) +
+                                     (1ull << F_YS) + (unsigned long long)ka + 4;
+    int sh = 0;
+    while (sh < 63 && (1ull << sh) < width) ++sh;
+    long long zlo, zhi;
+    box_range(bx, A, F_YS, zlo, zhi);
+    auto cell = [&](int2 p) { return (int)((unsigned long long)(z_at(p, A, F_YS) - zlo) >> sh) & (NC - 1); };
+    for (int k = threadIdx.x; k < n; k += T) atomicAdd(&cnt[cell(pts[k])], 1u);
+    __syncthreads();
+    const int per = NC / T;
+    unsigned sum = 0;
+    for (int r = 0; r < per; ++r) sum += cnt[threadIdx.x * per + r];
+    int total;
+    unsigned run = (unsigned)cta_scan_ex<T>((int)sum, s_warp, total);
+    for (int r = 0; r < per; ++r) {
+        const unsigned c = cnt[threadIdx.x * per + r];
+        cnt[threadIdx.x * per + r] = run;
+        run += c;
+    }
+    __syncthreads();
+    for (int k = threadIdx.x; k < n; k += T) ord[atomicAdd(&cnt[cell(pts[k])], 1u)] = (unsigned short)k;
+    __syncthreads();
+    const long long err = (1LL << F_YS) + ka + 4;
+    constexpr int L = T >= 32 ? 8 : 1;
+    for (int e = (part * T + (int)threadIdx.x) / L; e < n; e += T * parts / L) {
+        const int a = ord[e];
+        const int2 pa = pts[a];
+        const int q = cell(pa), q2 = (q + 1) & (NC - 1);
+        const int beg2 = q2 ? (int)cnt[q2 - 1] : 0;
+        const int n1 = (int)cnt[q] - e - 1, nn = n1 + (int)cnt[q2] - beg2;
+        if (*reinterpret_cast<volatile int *>(over)) break;   // the leaf is cut instead
+        for (int u = threadIdx.x % L; u < nn; u += L) {
+            const int b = ord[u < n1 ? e + 1 + u : beg2 + u - n1];
+            const int2 pb = pts[b];
+            // on the grid first: 0 <= dz < dx (B - A), widened
+            long long dx = (long long)pb.x - pa.x, dz = z_at(pb, A, F_YS) - z_at(pa, A, F_YS);
+            if (dx < 0) { dx = -dx; dz = -dz; }
+            if (dz < -err || (double)dz > (double)(dx + 1) * (double)(B - A) + (double)err) continue;
+            double s;
+            if (!slope_f32(f, a, b, s)) continue;
+            const double k = s * f.ratio * (double)(1LL << F_YS);
+            if (!(k >= (double)A && k < (double)B)) continue;
+            const int at = atomicAdd(nlist, 1);
+            if (at < HC) {
+                m.lkey[at] = order_of(s);
+                m.lden[at] = (unsigned)min(a, b) << 16 | (unsigned)max(a, b);
+            } else {
+                *over = 1;
+            }
+        }
+    }
+    __syncthreads();
+}
+
+// The narrowest window at the double slope s, as the float sweep computes it:
+// z = y - s x in double, w = z_hi - z_lo; ties take the lowest window.
+template <int T>
+__device__ __noinline__ void score_f32(const FloatSet &f, int n, int h, double s, unsigned char *wk, int wk_bytes,
+                                       unsigned char *gs, long long *s_red, double &w, double &t)
+{
+    int P = T;
+    while (P < n) P <<= 1;
+    auto key = [&](int k) { return k < n ? order_of(z_f32(f, k, s)) : D_MAX; };
+    long long *v = reinterpret_cast<long long *>(wk);
+    if (2 * P * 8 <= wk_bytes && P <= 16 * T) {
+        cta_fill_merge_sort_any(v, v + P, P, key);
+    } else {
+        long long *g = reinterpret_cast<long long *>(gs);
+        v = cta_sort_chunked<4 * T>(v, g, g + P, P, key);
+    }
+    long long bw = D_MAX;   // widths are >= 0: their bits order like them
+    int ba = 0x7fffffff;
+    for (int a = threadIdx.x; a + h - 1 < n; a += T) {
+        const long long d = order_of(__dsub_rn(of_order(v[a + h - 1]), of_order(v[a])));
+        if (d < bw) { bw = d; ba = a; }
+    }
+    if constexpr (T >= 32) {
+#pragma unroll
+        for (int d = 16; d >= 1; d >>= 1) {
+            const long long ow = __shfl_xor_sync(FULL, bw, d);
+            const int oa = __shfl_xor_sync(FULL, ba, d);
+            if (ow < bw || (ow == bw && oa < ba)) { bw = ow; ba = oa; }
+        }
+        if ((threadIdx.x & 31) == 0) {
+            s_red[2 * (threadIdx.x >> 5)] = bw;
+            s_red[2 * (threadIdx.x >> 5) + 1] = ba;
+        }
+        __syncthreads();
+        for (int q = 0; q < T / 32; ++q) {
+            const long long ow = s_red[2 * q];
+            const int oa = (int)s_red[2 * q + 1];
+            if (ow < bw || (ow == bw && oa < ba)) { bw = ow; ba = oa; }
+        }
+        __syncthreads();
+    }
+    const double zb = of_order(v[ba]), zt = of_order(v[ba + h - 1]);
+    w = zt - zb;
+    t = 0.5 * (zb + zt);
+    __syncthreads();
+}
+
+__device__ __forceinline__ bool candd_better(const CandD &a, const CandD &b)
+{
+    if (!a.valid) return false;
+    if (!b.valid) return true;
+    if (a.w != b.w) return a.w < b.w;
+    if (a.s != b.s) return a.s < b.s;
+    if (a.t != b.t) return a.t < b.t;
+    return a.pair < b.pair;
+}
+
+// Frame of a float set: centre and power-of-two scales that bring both axes
+// into the grid.  False (in every thread) when the set has values that are
+// not finite, no x range, or exponents so far apart that the scales would
+// leave the doubles' normal range: those are left to the sweep.
+template <int T>
+__device__ bool float_box(const float *x, const float *y, int n, FloatSet &f, Box &bx, long long *s_red)
+{
+    float xl = INFINITY, xh = -INFINITY, yl = INFINITY, yh = -INFINITY;
+    int bad = 0;
+    for (int k = threadIdx.x; k < n; k += T) {
+        const float u = x[k], v = y[k];
+        bad |= !(isfinite(u) && isfinite(v));
+        xl = fminf(xl, u); xh = fmaxf(xh, u);
+        yl = fminf(yl, v); yh = fmaxf(yh, v);
+    }
+    float *r = reinterpret_cast<float *>(s_red);
+    if constexpr (T >= 32) {
+#pragma unroll
+        for (int d = 16; d >= 1; d >>= 1) {
+            xl = fminf(xl, __shfl_xor_sync(FULL, xl, d)); xh = fmaxf(xh, __shfl_xor_sync(FULL, xh, d));
+            yl = fminf(yl, __shfl_xor_sync(FULL, yl, d)); yh = fmaxf(yh, __shfl_xor_sync(FULL, yh, d));
+        }
+        if ((threadIdx.x & 31) == 0) {
+            r[4 * (threadIdx.x >> 5)] = xl; r[4 * (threadIdx.x >> 5) + 1] = xh;
+            r[4 * (threadIdx.x >> 5) + 2] = yl; r[4 * (threadIdx.x >> 5) + 3] = yh;
+        }
+        bad = __syncthreads_or(bad);
+        for (int w = 0; w < T / 32; ++w) {
+            xl = fminf(xl, r[4 * w]); xh = fmaxf(xh, r[4 * w + 1]);
+            yl = fminf(yl, r[4 * w + 2]); yh = fmaxf(yh, r[4 * w + 3]);
+        }
+        __syncthreads();
+    }
+    const double dx = (double)xh - (double)xl, dy = (double)yh - (double)yl;
+    if (bad || !(dx > 1e-30) || !(dy > 1e-30) || dx > 1e30 || dy > 1e30) return false;
+    f.x = x;
+    f.y = y;
+    f.xc = 0.5 * ((double)xl + (double)xh);
+    f.yc = 0.5 * ((double)yl + (double)yh);
+    // |v - c| <= d / 2 < 2^(e - 1): scaled below 2^F_BITS
+    int ex, ey;
+    frexp(dx, &ex);
+    frexp(dy, &ey);
+    f.sx = ldexp(1.0, F_BITS + 1 - ex);
+    f.sy = ldexp(1.0, F_BITS + 1 - ey);
+    f.ratio = ldexp(1.0, ex - ey);
+    if (threadIdx.x == 0) {
+        bx.xc = bx.yc = bx.dh = 0;
+        bx.xlo = __double2int_rn(((double)xl - f.xc) * f.sx);
+        bx.xhi = __double2int_rn(((double)xh - f.xc) * f.sx);
+        bx.ylo = __double2int_rn(((double)yl - f.yc) * f.sy);
+        bx.yhi = __double2int_rn(((double)yh - f.yc) * f.sy);
+    }
+    return true;
+}
+
 // ------------------------------------------------------------------ exact score
 // The narrowest window at slope dy/dx: all projections sorted as exact
 // integers; ties take the lowest window.  wk: shared memory; gs: global
@@ -1209,6 +1461,8 @@ __device__ __noinline__ void line_pair(const int *pts, int n, int dy, int dx, un
 // ------------------------------------------------------------------ kernel
 struct DirectArgs {
     const short *x, *y;           // points of every set
+    const float *xf, *yf;         // points of a float set
+    int *done;                    // set to 1 once a float set's record is written
     const long long *off;         // set offsets (null: one set of n points)
     const int *hvec;              // order statistics per set (null: h)
     const int *sets;              // set indices in the order they are fitted (null: one set)
@@ -1326,10 +1580,11 @@ __device__ int cut_node(const DNode &nd, const long long *smp, int m, long long 
     return k;
 }
 
-template <int T, int G, int NB, int NBW, int PM, int LRUN, bool SP>
+template <int T, int G, int NB, int NBW, int PM, int LRUN, bool SP, bool F>
 __global__ void __launch_bounds__(T) k_direct(const DirectArgs A)
 {
     extern __shared__ __align__(16) unsigned char dsm[];
+    using P_t = std::conditional_t<F, int2, int>;
     constexpr int GROUPS = T / G;
     constexpr int NS = T < 512 ? 512 : T;   // sampled slopes
     constexpr int LC = LRUN + PM;
@@ -1372,15 +1627,20 @@ __global__ void __launch_bounds__(T) k_direct(const DirectArgs A)
         } else if (turn) {
             return;
         }
-        const short *x = A.x + base, *y = A.y + base;
-        int *pts_s = reinterpret_cast<int *>(dsm + sizeof(Shared));
-        int *pts = SP ? pts_s : m.pts;
-        unsigned char *wk = dsm + sizeof(Shared) + (SP ? ((4 * n + 15) & ~15) : 0);
+        [[maybe_unused]] const short *x = A.x + base, *y = A.y + base;
+        P_t *pts = SP ? reinterpret_cast<P_t *>(dsm + sizeof(Shared)) : reinterpret_cast<P_t *>(m.pts);
+        unsigned char *wk = dsm + sizeof(Shared) + (SP ? (((int)sizeof(P_t) * n + 15) & ~15) : 0);
         const int wk_bytes = (int)smem_size() - (int)(wk - dsm);
         int *hist = reinterpret_cast<int *>(wk) + g.id * NB, *histw = reinterpret_cast<int *>(wk);
 
         // ---------------------------------------------------------- box, centred points
-        {
+        FloatSet fs{};
+        if constexpr (F) {
+            if (!float_box<T>(A.xf, A.yf, n, fs, S.bx, S.red)) return;   // left to the sweep
+            for (int k = (SP ? 0 : (int)rank * T) + (int)threadIdx.x; k < n; k += SP ? T : T * (int)C)
+                pts[k] = make_int2(__double2int_rn(((double)A.xf[k] - fs.xc) * fs.sx),
+                                   __double2int_rn(((double)A.yf[k] - fs.yc) * fs.sy));
+        } else {
             int xl = 0x7fffffff, xh = -0x7fffffff, yl = 0x7fffffff, yh = -0x7fffffff;
             for (int k = threadIdx.x; k < n; k += T) {
                 const int xv = x[k], yv = y[k];
@@ -1412,6 +1672,7 @@ __global__ void __launch_bounds__(T) k_direct(const DirectArgs A)
         }
         team_sync();
         const int algo = n <= A.plain_max ? LMS_ALGO_PLAIN : n >= A.bnb_min ? LMS_ALGO_BNB : A.algo;
+        if constexpr (!F) {
         if (S.bx.xlo == S.bx.xhi) {
             // every x equal: the window at slope 0
             if (rank == 0) {
@@ -1421,6 +1682,7 @@ __global__ void __launch_bounds__(T) k_direct(const DirectArgs A)
             }
             team_sync();
             continue;
+        }
         }
         // a lower bound of the x-span of any h points: narrowest window of h
         // over the histogram of x, less its two end bins
@@ -1436,7 +1698,14 @@ __global__ void __launch_bounds__(T) k_direct(const DirectArgs A)
         __syncthreads();
         const Box bx = S.bx;
         const int yr = bx.yhi - bx.ylo, xr = bx.xhi - bx.xlo;
-        const long long kmax = ((long long)yr + 1) << 32;   // above every pair's slope
+        // above every pair's slope; float sets leave steeper ones to the bound below
+        const long long kmax = F ? F_KMAX : ((long long)yr + 1) << 32;
+
+        // Float sets: w at a slope differs by at most (1 + |s|) steps from w of the
+        // grid points.  An upper bound is raised by that much, and an interval is
+        // tested against the upper bound raised once more.
+        auto grid_key = [&](double s) { return (long long)floor(s * fs.ratio * (double)(1LL << F_YS)); };
+        auto grid_err = [](long long K) { return F ? (1LL << F_YS) + (K < 0 ? -K : K) + 4 : 0LL; };
 
         // ---------------------------------------------------------- sampled slopes (the same in every CTA)
         {
@@ -1445,9 +1714,16 @@ __global__ void __launch_bounds__(T) k_direct(const DirectArgs A)
                 const int i = (int)__umulhi(u, (unsigned)n);
                 int j = (int)__umulhi(v, (unsigned)(n - 1));
                 j += j >= i;
-                int dy, dx;
-                if (!pair_slope(pts[i], pts[j], dy, dx)) return D_MAX;
-                return slope_key(dy, dx);
+                if constexpr (F) {
+                    double v;
+                    if (!slope_f32(fs, i, j, v)) return D_MAX;
+                    v *= fs.ratio * (double)(1LL << F_YS);
+                    return fabs(v) < (double)(F_KMAX - 1) ? (long long)floor(v) : D_MAX;
+                } else {
+                    int dy, dx;
+                    if (!pair_slope(pts[i], pts[j], dy, dx)) return D_MAX;
+                    return slope_key(dy, dx);
+                }
             };
             long long *s = reinterpret_cast<long long *>(wk);
             cta_fill_merge_sort_any(s, s + NS, NS, sample);
@@ -1473,7 +1749,7 @@ __global__ void __launch_bounds__(T) k_direct(const DirectArgs A)
                 if (!A.pred) return false;
                 const float v = *A.pred;
                 if (!(fabsf(v) < 16000.0f)) return false;
-                K = (long long)((double)v * 4294967296.0);
+                K = (long long)((double)v * 4294967296.0);   // float sets have no prediction
             }
             return K > -kmax && K < kmax;
         };
@@ -1482,6 +1758,7 @@ __global__ void __launch_bounds__(T) k_direct(const DirectArgs A)
             long long K, lower = D_MAX;
             if (seed(q, K)) {
                 lower = ub_at<G, NB>(g, pts, n, h, K, D_MAX, bx, hist, 1, 0, true);
+                if (lower < D_MAX) lower += grid_err(K);
                 if (g.lane == 0 && lower < D_MAX) atomicMin(&st->ub, lower);
             }
             if (g.lane == 0) m.ans[q].t0 = lower;   // the coarse width
@@ -1504,7 +1781,7 @@ __global__ void __launch_bounds__(T) k_direct(const DirectArgs A)
                 if (!seed(S.keep[i], K)) return;
                 const long long u = gr.first(__ldcg(&st->ub));   // others lower it meanwhile: one value for the group
                 const long long w = ub_at<GG, decltype(nb)::value>(gr, pts, n, h, K, u, bx, hs, 1, 0);
-                if (gr.lane == 0 && w < u) atomicMin(&st->ub, w);
+                if (gr.lane == 0 && w < D_MAX / 2 && w + grid_err(K) < u) atomicMin(&st->ub, w + grid_err(K));
             };
             if (C > 1 && ns <= (int)C * WIDE_ITEMS) {
                 for (int i = rank; i < ns; i += C) refine(gw, std::integral_constant<int, NBW>(), histw, i);
@@ -1524,10 +1801,11 @@ __global__ void __launch_bounds__(T) k_direct(const DirectArgs A)
         }
         // the plan: the same values in every thread of the team
         int mode = M_TREE, P = Q + 1, cur = 0, par = 0, lpar = 0, ppar = 0;
-        int top = 0, etop = 0, nleaf = 0, lf0 = 0, lfn = 0, nx = 0, err = 0, regrown = 0;
+        int top = 0, etop = 0, nleaf = 0, lf0 = 0, lfn = 0, nx = 0, err = 0, regrown = 0, scored = 0;
         bool flush = false;
         long long ux = D_MAX, uxl = D_MAX, bkey = D_MAX;
         Cand best = cand_empty();
+        CandD bestd{};
         team_sync();
         for (int phase = 0; mode != M_DONE; ++phase) {
             DNode *work = S.work[cur], *next = S.work[cur ^ 1];
@@ -1538,12 +1816,20 @@ __global__ void __launch_bounds__(T) k_direct(const DirectArgs A)
                 auto test = [&](auto &gr, auto nb, int *hs, int k) {
                     constexpr int GG = std::remove_reference_t<decltype(gr)>::SIZE;
                     const DNode &nd = work[k];
-                    const long long ka = ev ? __ldcg(&m.ev[nd.a]) : nd.a;
-                    const long long kb = ev ? __ldcg(&m.ev[nd.b - 1]) + 1 : nd.b;
-                    const long long U = min(gr.first(__ldcg(&st->ub)), ka > bkey ? uxl : ux);
+                    long long ka = ev ? __ldcg(&m.ev[nd.a]) : nd.a;
+                    long long kb = ev ? __ldcg(&m.ev[nd.b - 1]) + 1 : nd.b;
+                    const bool right = F && !ev ? bestd.valid && ka > grid_key(bestd.s) + 1 : ka > bkey;
+                    long long U = min(gr.first(__ldcg(&st->ub)), right ? uxl : ux);
+                    if constexpr (F) {
+                        if (ev) {
+                            ka = grid_key(of_order(ka)) - 1;
+                            kb = grid_key(of_order(kb - 1)) + 2;
+                        }
+                        if (U >= 0 && U < D_MAX / 2) U += max(grid_err(ka), grid_err(kb)) + 4;
+                    }
                     long long t0 = nd.t0, t1 = nd.t1;
                     bool keep;
-                    if ((!ev && nd.est < 0.0f) || steep_above(ka, kb, bx.dh, yr, U)) keep = false;
+                    if ((!ev && nd.est < 0.0f) || (!F && steep_above(ka, kb, bx.dh, yr, U))) keep = false;
                     else
                         keep = may_hold<GG, decltype(nb)::value>(gr, pts, n, h, ka, kb, U, ev ? U >> 18 : U >> 12, bx,
                                                                  hs, t0, t1);
@@ -1577,10 +1863,11 @@ __global__ void __launch_bounds__(T) k_direct(const DirectArgs A)
                     constexpr int GG = std::remove_reference_t<decltype(gr)>::SIZE;
                     const DNode &nd = work[S.keep[i]];
                     if (ev && nd.b - nd.a == 1) return;
-                    const long long K = ev ? __ldcg(&m.ev[(nd.a + nd.b) >> 1]) : nd.a + ((nd.b - nd.a) >> 1);
+                    long long K = ev ? __ldcg(&m.ev[(nd.a + nd.b) >> 1]) : nd.a + ((nd.b - nd.a) >> 1);
+                    if (F && ev) K = grid_key(of_order(K));
                     const long long ub = gr.first(__ldcg(&st->ub));
                     const long long w = ub_at<GG, decltype(nb)::value>(gr, pts, n, h, K, ub, bx, hs, nd.t0, nd.t1);
-                    if (gr.lane == 0 && w < ub) atomicMin(&st->ub, w);
+                    if (gr.lane == 0 && w < D_MAX / 2 && w + grid_err(K) < ub) atomicMin(&st->ub, w + grid_err(K));
                 };
                 if (ns > 0) {
                     if (C > 1 && ns <= (int)C * WIDE_ITEMS) {
@@ -1597,7 +1884,7 @@ __global__ void __launch_bounds__(T) k_direct(const DirectArgs A)
                     if (nd.b > -(D_GUARD - 1) && nd.a <= -D_GUARD) return false;
                     if (nd.b - nd.a == 1) return true;
                     if (nd.force > 0) return false;
-                    return nd.est <= sh.leaf || fractions(nd.a, nd.b, xr) <= LEAF_FRACTIONS;
+                    return nd.est <= sh.leaf || (!F && fractions(nd.a, nd.b, xr) <= LEAF_FRACTIONS);
                 };
                 const int pers = (ns + T - 1) / T;
                 const int i0 = min(ns, (int)threadIdx.x * pers), i1 = min(ns, i0 + pers);
@@ -1671,8 +1958,12 @@ __global__ void __launch_bounds__(T) k_direct(const DirectArgs A)
                 const int parts = max(1, (int)C / lfn);
                 for (int l = rank; l < lfn * parts; l += C) {
                     const DNode &lf = S.leaf[lf0 + l / parts];
-                    list_pairs<T>(pts, n, lf.a, lf.b, bx, NC, wk, S.warp_a, m, &st->nlist[lpar], &st->over[lpar], sh.HC,
-                                  l % parts, parts);
+                    if constexpr (F)
+                        list_pairs_f32<T>(pts, n, lf.a, lf.b, bx, fs, NC, wk, S.warp_a, m, &st->nlist[lpar],
+                                          &st->over[lpar], sh.HC, l % parts, parts);
+                    else
+                        list_pairs<T>(pts, n, lf.a, lf.b, bx, NC, wk, S.warp_a, m, &st->nlist[lpar], &st->over[lpar],
+                                      sh.HC, l % parts, parts);
                 }
                 team_sync();
                 const bool over = __ldcg(&st->over[lpar]) != 0;
@@ -1693,8 +1984,13 @@ __global__ void __launch_bounds__(T) k_direct(const DirectArgs A)
                     } else {
                         int P2 = T;
                         while (P2 < nn) P2 <<= 1;
-                        cta_fill_merge_sort_any(s, s + P2, P2,
-                                                [&](int k) { return k < nn ? __ldcg(&m.lkey[k]) : D_MAX; });
+                        auto key = [&](int k) { return k < nn ? __ldcg(&m.lkey[k]) : D_MAX; };
+                        if (16 * P2 <= wk_bytes) {
+                            cta_fill_merge_sort_any(s, s + P2, P2, key);
+                        } else {
+                            long long *gk = reinterpret_cast<long long *>(gsort);
+                            s = cta_sort_chunked<4 * T>(s, gk, gk + P2, P2, key);
+                        }
                         for (int k = threadIdx.x; k < nn; k += T) {
                             m.ev[k] = s[k];
                             const long long v = __ldcg(&m.lkey[k]);
@@ -1741,7 +2037,7 @@ __global__ void __launch_bounds__(T) k_direct(const DirectArgs A)
                         lf0 = nleaf = 0;
                         flush = false;
                     }
-                } else if (lfn > 1 && regrown < 2 && lfn <= PM && lfn == nleaf) {
+                } else if (lfn > 1 && regrown < (F ? 8 : 2) && lfn <= PM && lfn == nleaf) {
                     // their expected pairs were too low: cut them once more
                     for (int j = threadIdx.x; j < lfn; j += T) {
                         DNode nd = S.leaf[j];
@@ -1773,7 +2069,7 @@ __global__ void __launch_bounds__(T) k_direct(const DirectArgs A)
                 }
                 team_sync();
                 if (over && P == 0) {
-                    if (phase > PHASES_MAX) err = 1;
+                    if (phase > (F ? F_PHASES : PHASES_MAX)) err = 1;
                     mode = err ? M_DONE : M_PAIRS;
                     continue;
                 }
@@ -1784,6 +2080,36 @@ __global__ void __launch_bounds__(T) k_direct(const DirectArgs A)
                 }
             } else {
                 // ------------------------------------------------ exact scores
+                if constexpr (F) {
+                    scored += nx;
+                    if (scored > F_SCORES) err = 1;
+                    for (int k = rank; k < nx && !err; k += C) {
+                        CandD c;
+                        c.s = of_order(__ldcg(&m.ev[S.xl[k]]));
+                        c.pair = __ldcg(&m.evd[S.xl[k]]);
+                        c.valid = 1;
+                        score_f32<T>(fs, n, h, c.s, wk, wk_bytes, gsort, S.red, c.w, c.t);
+                        if (threadIdx.x == 0) reinterpret_cast<CandD *>(m.xres)[k] = c;
+                    }
+                    team_sync();
+                    for (int k = 0; k < nx && !err; ++k) {
+                        const CandD *q = reinterpret_cast<const CandD *>(m.xres) + k;
+                        CandD c;
+                        c.w = __ldcg(&q->w);
+                        c.s = __ldcg(&q->s);
+                        c.t = __ldcg(&q->t);
+                        c.pair = __ldcg(&q->pair);
+                        c.valid = 1;
+                        if (candd_better(c, bestd)) bestd = c;
+                    }
+                    // the true width, rounded up, bounds the rest; nothing right of a width of 0 is better
+                    if (bestd.valid) {
+                        const double u = bestd.w * fs.sy * (double)(1LL << F_YS);
+                        ux = u < 4e18 ? (long long)u + 2 : D_MAX;
+                        uxl = bestd.w == 0.0 ? -1 : ux;
+                        bkey = order_of(bestd.s);
+                    }
+                } else {
                 for (int k = rank; k < nx; k += C) {
                     const int dx = (int)__ldcg(&m.evd[S.xl[k]]), dy = dy_of(__ldcg(&m.ev[S.xl[k]]), dx);
                     Cand c;
@@ -1830,13 +2156,14 @@ __global__ void __launch_bounds__(T) k_direct(const DirectArgs A)
                     uxl = (r % best.dx) ? ux : ux - 1;
                     bkey = slope_key(best.dy, best.dx);
                 }
+                }
                 nx = 0;
                 P = 0;
                 __syncthreads();
             }
             // ---------------------------------------------------- the next phase
             const bool was_tree = mode == M_TREE;
-            if (err || phase > PHASES_MAX) {
+            if (err || phase > (F ? F_PHASES : PHASES_MAX)) {
                 err = 1;
                 mode = M_DONE;
             } else if (nx > 0) {
@@ -1872,7 +2199,47 @@ __global__ void __launch_bounds__(T) k_direct(const DirectArgs A)
                 mode = M_DONE;
             }
         }
-        if (rank == 0 && threadIdx.x == 0) write_result(A.out + set, best, algo, err | __ldcg(&st->bad));
+        if constexpr (F) {
+            // the smallest index pair with the best slope: its pairs listed once more
+            if (rank == 0 && threadIdx.x == 0) st->nlist[lpar] = st->over[lpar] = 0;
+            team_sync();
+            if (bestd.valid && !err) {
+                int NC = T;
+                while (NC < n && NC < CELLS_MAX) NC <<= 1;
+                const long long K = grid_key(bestd.s);
+                list_pairs_f32<T>(pts, n, K - 1, K + 2, bx, fs, NC, wk, S.warp_a, m, &st->nlist[lpar], &st->over[lpar],
+                                  sh.HC, (int)rank, (int)C);
+            }
+            team_sync();
+            if (rank == 0 && bestd.valid && !err) {
+                const int nn = min(__ldcg(&st->nlist[lpar]), sh.HC);
+                int first = 0x7fffffff, last = 0;
+                for (int k = threadIdx.x; k < nn; k += T)
+                    if (__ldcg(&m.lkey[k]) == order_of(bestd.s)) first = min(first, (int)__ldcg(&m.lden[k]));
+                cta_min_max_i<T>(first, last, S.warp_a, S.warp_b);
+                if (__ldcg(&st->over[lpar])) err = 1;
+                else bestd.pair = (unsigned)first;
+            }
+            // slopes beyond the tree's range must be out of reach
+            const long long U = min(__ldcg(&st->ub), ux);
+            const bool tails = steep_above_at(F_KMAX, bx.dh, yr, U < D_MAX / 2 ? U + grid_err(F_KMAX) : D_MAX);
+            if (rank == 0 && threadIdx.x == 0 && !err && tails && bestd.valid) {
+                lms_result r;
+                r.w_num = r.w_den = r.s_num = r.s_den = r.t_num = r.t_den = 0;
+                r.theta1 = bestd.s;
+                r.theta2 = bestd.t;
+                const double half = 0.5 * bestd.w;
+                r.med_sq = half * half;
+                r.i = (int)(bestd.pair >> 16);
+                r.j = (int)(bestd.pair & 0xffffu);
+                r.status = LMS_OK;
+                r.algorithm = algo;
+                *A.out = r;
+                *A.done = 1;
+            }
+        } else {
+            if (rank == 0 && threadIdx.x == 0) write_result(A.out + set, best, algo, err | __ldcg(&st->bad));
+        }
         team_sync();
     }
 }
@@ -1880,10 +2247,10 @@ __global__ void __launch_bounds__(T) k_direct(const DirectArgs A)
 
 // ------------------------------------------------------------------ host
 // The kernel's shapes: for one fit in a cluster by its size, and for batches.
-template <int T_, int G_, int NB_, int NBW_, int PM_, int LRUN_, bool SP_>
+template <int T_, int G_, int NB_, int NBW_, int PM_, int LRUN_, bool SP_, bool F_ = false>
 struct Shape {
-    static constexpr int T = T_, PM = PM_, LC = LRUN_ + PM_, NS = T_ < 512 ? 512 : T_;
-    static constexpr auto kernel = k_direct<T_, G_, NB_, NBW_, PM_, LRUN_, SP_>;
+    static constexpr int T = T_, PM = PM_, LC = LRUN_ + PM_, NS = T_ < 512 ? 512 : T_, PT = F_ ? 8 : 4;
+    static constexpr auto kernel = k_direct<T_, G_, NB_, NBW_, PM_, LRUN_, SP_, F_>;
     // shared memory of a CTA whose largest set has n points
     static size_t smem(int n, int HC)
     {
@@ -1896,7 +2263,7 @@ struct Shape {
         wk = std::max(wk, pairs_bytes((int)NC, n));
         wk = std::max(wk, 16 * P2);
         wk = std::max(wk, std::min<size_t>(8 * P, 64 * (size_t)T));   // 32-bit exact sort, or its chunks
-        return sizeof(DShared<NS, PM, LC>) + (SP_ ? ((4 * (size_t)n + 15) & ~(size_t)15) : 0) + wk;
+        return sizeof(DShared<NS, PM, LC>) + (SP_ ? ((PT * (size_t)n + 15) & ~(size_t)15) : 0) + wk;
     }
     static TeamShape team(int nmax, int C, int HC, float leaf)
     {
@@ -1908,8 +2275,8 @@ struct Shape {
         t.HC = HC;
         t.Q = std::min(PM, 128) - 1;
         t.leaf = leaf;
-        t.ptsn = SP_ ? 0 : nmax;
-        t.sortw = (long long)(16 * P);
+        t.ptsn = SP_ ? 0 : (long long)nmax * (PT / 4);
+        t.sortw = 16LL * std::max<long long>(P, HC);
         t.C = C;
         return t;
     }
@@ -1917,6 +2284,8 @@ struct Shape {
 using Small = Shape<512, 32, 1024, 4096, 256, 64, true>;
 using Mid = Shape<1024, 128, 2048, 4096, 256, 64, true>;
 using Large = Shape<1024, 256, 4096, 8192, 128, 64, false>;
+using FloatSmall = Shape<512, 32, 1024, 4096, 256, 64, true, true>;
+using FloatMid = Shape<1024, 128, 2048, 4096, 256, 64, true, true>;
 using Batch = Shape<256, 32, 1024, 1024, 64, 32, true>;
 
 struct Single {
@@ -1939,6 +2308,21 @@ Single single_of(int n)
     } else {
         s.shape = Large::team(n, C, 4096, 1024.0f);
         s.smem = Large::smem(n, 4096);
+    }
+    return s;
+}
+
+Single float_single_of(int n)
+{
+    Single s{};
+    s.variant = n <= 2048 ? 0 : 1;
+    const int C = 16;
+    if (s.variant == 0) {
+        s.shape = FloatSmall::team(n, C, 4096, 256.0f);
+        s.smem = FloatSmall::smem(n, 4096);
+    } else {
+        s.shape = FloatMid::team(n, C, 16384, 256.0f);
+        s.smem = FloatMid::smem(n, 4096);   // a longer list is sorted in chunks
     }
     return s;
 }
@@ -1967,6 +2351,13 @@ cudaError_t launch_cluster(const DirectArgs &a, size_t smem, cudaStream_t st)
 
 }  // namespace
 
+// Float sets: up to 4096 points.  The grid's error (a few 2^-30 of the axes)
+// keeps every slope alive whose width is within about 1e-5 of the optimum:
+// tens of slopes up to here (0.49 ms against 1.29 at n = 2048, 0.64 - 1.0
+// against 2.5 - 2.9 at 4096), thousands above (n = 8192: 1.7 - 9.7 ms against
+// 9.2 - 10.3), each scored by a sort.
+bool direct_f32_ok(int n, int h) { return n >= 16 && n <= 4096 && (long long)h * 4 >= n; }
+
 bool direct_ok(int n, int h) { return n >= 2 && n <= 65536 && (long long)h * 8 >= n; }
 
 size_t direct_bytes(int n) { return (size_t)d_up(team_bytes(single_of(n).shape)); }
@@ -1992,6 +2383,31 @@ cudaError_t launch_direct(const short *x, const short *y, int n, int h, int algo
     if (s.variant == 0) return launch_cluster<Small>(a, s.smem, st);
     if (s.variant == 1) return launch_cluster<Mid>(a, s.smem, st);
     return launch_cluster<Large>(a, s.smem, st);
+}
+
+// ---------------------------------------------------------------- float sets
+size_t direct_f32_bytes(int n) { return (size_t)d_up(team_bytes(float_single_of(n).shape)); }
+
+cudaError_t launch_direct_f32(const float *x, const float *y, int n, int h, int algo, lms_result *out, int *done,
+                              void *mem, cudaStream_t st)
+{
+    const Single s = float_single_of(n);
+    DirectArgs a = {};
+    a.xf = x;
+    a.yf = y;
+    a.n = n;
+    a.h = h;
+    a.nsets = 1;
+    a.algo = algo;
+    a.bnb_min = 0x7fffffff;
+    a.out = out;
+    a.done = done;
+    a.mem = static_cast<unsigned char *>(mem);
+    a.shape = s.shape;
+    cudaError_t e = cudaMemsetAsync(done, 0, sizeof(int), st);
+    if (e != cudaSuccess) return e;
+    StageTimer _t(STAGE_DIRECT, st);
+    return s.variant == 0 ? launch_cluster<FloatSmall>(a, s.smem, st) : launch_cluster<FloatMid>(a, s.smem, st);
 }
 
 // ---------------------------------------------------------------- many sets

@@ -131,6 +131,7 @@ struct SweepPlan {
     bool resplit;
     long long *bnd2;           // [BND_MAX] boundaries of the kept events' buckets
     unsigned *base2;           // [BND_MAX + 1] their starts
+    const int *skip = nullptr; // when not null and set (device), the fit is done already: its kernels return at once
     int *meta2;                // [16] their nbnd, P2 and oversize count (layout of meta)
 };
 constexpr int RESPLIT_PER = 4096;    // kept events per bucket of a resplit pass
@@ -203,6 +204,13 @@ size_t direct_bytes(int n);   // device scratch of one fit
 // predicted slope on the device, or null.
 cudaError_t launch_direct(const short *x, const short *y, int n, int h, int algo, const float *pred, lms_result *out,
                           void *mem, cudaStream_t st);
+// One float fit, tried before the sweep: *done (device) becomes 1 once its
+// record is written, 0 when the set is left to the sweep (not finite, no x
+// range, slopes out of the grid's reach, too many near-ties).
+bool direct_f32_ok(int n, int h);
+size_t direct_f32_bytes(int n);
+cudaError_t launch_direct_f32(const float *x, const float *y, int n, int h, int algo, lms_result *out, int *done,
+                              void *mem, cudaStream_t st);
 // Many sets of at most nmax <= DIRECT_BATCH_MAX points, one CTA each: sets
 // (device) lists the set indices in the order they are handed out.
 constexpr int DIRECT_BATCH_MAX = 4096;

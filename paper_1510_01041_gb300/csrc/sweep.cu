@@ -128,8 +128,9 @@ __global__ void k_pack(const short *__restrict__ x, const short *__restrict__ y,
 
 // ---------------------------------------------------------------- sample
 template <class G>
-__global__ void k_sample(const void *__restrict__ pts, int n, long long npairs, int S, long long *__restrict__ out)
+__global__ void k_sample(const int *skip, const void *__restrict__ pts, int n, long long npairs, int S, long long *__restrict__ out)
 {
+    if (skip && *skip) return;
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= S) return;
     const unsigned long long r = mix64(0x5851F42D4C957F2Dull + (unsigned long long)k * 0x9E3779B97F4A7C15ull);
@@ -145,8 +146,9 @@ __global__ void k_sample(const void *__restrict__ pts, int n, long long npairs, 
 // chunks are merged in one pass by ranking.
 constexpr int SAMPLE_CH = 8192;
 
-__global__ void __launch_bounds__(1024) k_sort_chunks(long long *__restrict__ keys, int S)
+__global__ void __launch_bounds__(1024) k_sort_chunks(const int *skip, long long *__restrict__ keys, int S)
 {
+    if (skip && *skip) return;
     extern __shared__ __align__(16) unsigned char smem[];
     long long *s = reinterpret_cast<long long *>(smem);
     const int P = S < SAMPLE_CH ? S : SAMPLE_CH;
@@ -160,9 +162,10 @@ __global__ void __launch_bounds__(1024) k_sort_chunks(long long *__restrict__ ke
 // chunks before c and < it in the chunks after (a stable order, every
 // position taken once).  The binary searches over the chunks are
 // independent and run together.
-__global__ void __launch_bounds__(256) k_merge_chunks(const long long *__restrict__ src, long long *__restrict__ dst,
+__global__ void __launch_bounds__(256) k_merge_chunks(const int *skip, const long long *__restrict__ src, long long *__restrict__ dst,
                                                       int S)
 {
+    if (skip && *skip) return;
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= S) return;
     const int nch = S / SAMPLE_CH, c = k / SAMPLE_CH;
@@ -196,10 +199,11 @@ __global__ void __launch_bounds__(256) k_merge_chunks(const long long *__restric
 // KEY_INF to the power of two P2 > nbnd.
 // bcount (optional): the number of keys the buckets will hold; then B is
 // lowered to about *bcount / bper buckets.
-__global__ void __launch_bounds__(1024) k_splitters(const long long *__restrict__ sorted, int S, int B,
+__global__ void __launch_bounds__(1024) k_splitters(const int *skip, const long long *__restrict__ sorted, int S, int B,
                                                     long long *__restrict__ bnd, int *__restrict__ meta,
                                                     const int *__restrict__ bcount = nullptr, int bper = 1)
 {
+    if (skip && *skip) return;
     extern __shared__ long long s_q[];   // the B - 1 quantiles (at most BND_MAX / 2)
     __shared__ int s_m;
     __shared__ int s_scan[1024];
@@ -274,7 +278,7 @@ __global__ void __launch_bounds__(1024) k_splitters(const long long *__restrict_
 // restricted fit lists its pairs with the band scan below; the scatter then
 // places the list, k_scatter_list, whatever the order.)
 template <bool SCATTER, class G>
-__global__ void __launch_bounds__(CNT_THREADS) k_bucket_pairs(const void *__restrict__ pts, int n,
+__global__ void __launch_bounds__(CNT_THREADS) k_bucket_pairs(const int *skip, const void *__restrict__ pts, int n,
                                                               const long long *__restrict__ bnd,
                                                               const int *__restrict__ meta,
                                                               unsigned *__restrict__ hist,
@@ -282,6 +286,7 @@ __global__ void __launch_bounds__(CNT_THREADS) k_bucket_pairs(const void *__rest
                                                               unsigned *__restrict__ ev,
                                                               const unsigned char *__restrict__ keep)
 {
+    if (skip && *skip) return;
     extern __shared__ __align__(16) unsigned char smem[];
     long long *s_bnd = reinterpret_cast<long long *>(smem);
     unsigned *s_cnt = reinterpret_cast<unsigned *>(smem + BND_MAX * sizeof(long long));
@@ -824,9 +829,10 @@ __global__ void k_sample_counts(const long long *__restrict__ sorted, int S, con
 }
 
 // Per bucket: exclusive prefix over CTAs (in place) and the bucket total.
-__global__ void k_bucket_prefix(unsigned *__restrict__ hist, int C, const int *__restrict__ meta,
+__global__ void k_bucket_prefix(const int *skip, unsigned *__restrict__ hist, int C, const int *__restrict__ meta,
                                 unsigned *__restrict__ total)
 {
+    if (skip && *skip) return;
     const int b = blockIdx.x * blockDim.x + threadIdx.x;
     if (b > meta[0]) return;
     unsigned run = 0;
@@ -840,9 +846,10 @@ __global__ void k_bucket_prefix(unsigned *__restrict__ hist, int C, const int *_
 
 // Exclusive scan of bucket totals (in place, NB <= BND_MAX); base[NB] = E.
 // copy (optional): receives the bucket starts too (the list scatter's cursors).
-__global__ void __launch_bounds__(1024) k_bucket_scan(unsigned *__restrict__ base, const int *__restrict__ meta,
+__global__ void __launch_bounds__(1024) k_bucket_scan(const int *skip, unsigned *__restrict__ base, const int *__restrict__ meta,
                                                       unsigned *__restrict__ copy = nullptr)
 {
+    if (skip && *skip) return;
     __shared__ unsigned s[1024];
     const int NB = meta[0] + 1;
     const int per = (NB + 1023) / 1024;
@@ -1012,11 +1019,12 @@ __device__ bool sort_bucket_words(const void *__restrict__ xy, const unsigned *s
 // SEG_CAP events are listed for k_segsort_big.  A bucket holding a single
 // slope only needs its smallest pair moved to the front.
 template <class G>
-__global__ void __launch_bounds__(1024) k_segsort(const void *__restrict__ xy, unsigned *__restrict__ ev,
+__global__ void __launch_bounds__(1024) k_segsort(const int *skip, const void *__restrict__ xy, unsigned *__restrict__ ev,
                                                   const unsigned *__restrict__ base,
                                                   const long long *__restrict__ bnd, int *__restrict__ meta,
                                                   int *__restrict__ oversize)
 {
+    if (skip && *skip) return;
     extern __shared__ __align__(16) unsigned char smem[];
     long long *s_key = reinterpret_cast<long long *>(smem);
     unsigned *s_ev = reinterpret_cast<unsigned *>(smem + SEG_CAP * sizeof(long long));
@@ -1239,12 +1247,13 @@ __device__ void sort_big_merge(const void *__restrict__ xy, unsigned *A, unsigne
 }
 
 template <class G>
-__global__ void __launch_bounds__(1024) k_segsort_big(const void *__restrict__ xy, unsigned *__restrict__ ev,
+__global__ void __launch_bounds__(1024) k_segsort_big(const int *skip, const void *__restrict__ xy, unsigned *__restrict__ ev,
                                                       unsigned *__restrict__ ev2,
                                                       const unsigned *__restrict__ base,
                                                       const int *__restrict__ meta,
                                                       const int *__restrict__ oversize)
 {
+    if (skip && *skip) return;
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ long long s_spl[SB_MAX];
     __shared__ unsigned s_cnt[SB_MAX + 1], s_cur[SB_MAX];
@@ -1364,9 +1373,10 @@ __device__ unsigned snap_group_start(const unsigned *__restrict__ ev, const unsi
 // Range r covers the events [s(E r / W), s(E (r + 1) / W)), s = the snap to
 // a group start below: equal event counts up to the group granularity.  One
 // warp per range.
-__global__ void k_plan(const unsigned *__restrict__ ev, const unsigned *__restrict__ base,
+__global__ void k_plan(const int *skip, const unsigned *__restrict__ ev, const unsigned *__restrict__ base,
                        const int *__restrict__ meta, int W, unsigned *__restrict__ range)
 {
+    if (skip && *skip) return;
     const int r = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
     if (r >= W) return;
     const int NB = meta[0] + 1;
@@ -1399,8 +1409,9 @@ __global__ void k_snap_ranges(const unsigned *__restrict__ ev, const unsigned *_
 // the previous range already covers, and the ranges become disjoint, so every
 // event is swept exactly once (k_sweep checks the total).  One CTA, in
 // chunks of consecutive bounds per thread.
-__global__ void __launch_bounds__(1024) k_monotone_ranges(unsigned *__restrict__ range, int count)
+__global__ void __launch_bounds__(1024) k_monotone_ranges(const int *skip, unsigned *__restrict__ range, int count)
 {
+    if (skip && *skip) return;
     __shared__ unsigned s_warp[32];
     const int per = (count + blockDim.x - 1) / blockDim.x;
     const int k0 = threadIdx.x * per, k1 = min(count, k0 + per);
@@ -2540,14 +2551,14 @@ const long long *sorted_sample(const SweepPlan &p)
 
 // Sorts S sampled keys (a power of two, SORT_CHUNK .. 16 SAMPLE_CH) held in
 // keys, scratch beside; returns the array that holds the sorted keys.
-static long long *sort_sample(long long *keys, long long *scratch, int S, cudaStream_t st)
+static long long *sort_sample(const int *skip, long long *keys, long long *scratch, int S, cudaStream_t st)
 {
     const int P = std::min(S, SAMPLE_CH);
     const size_t smem = (size_t)2 * P * 8;
     cudaFuncSetAttribute(k_sort_chunks, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    { StageTimer _t(STAGE_SAMPLE_SORT, st); k_sort_chunks<<<S / P, 1024, smem, st>>>(keys, S); }
+    { StageTimer _t(STAGE_SAMPLE_SORT, st); k_sort_chunks<<<S / P, 1024, smem, st>>>(skip, keys, S); }
     if (S <= SAMPLE_CH) return keys;
-    { StageTimer _t(STAGE_SAMPLE_SORT, st); k_merge_chunks<<<(S + 255) / 256, 256, 0, st>>>(keys, scratch, S); }
+    { StageTimer _t(STAGE_SAMPLE_SORT, st); k_merge_chunks<<<(S + 255) / 256, 256, 0, st>>>(skip, keys, scratch, S); }
     return scratch;
 }
 
@@ -2555,13 +2566,13 @@ template <class G>
 static cudaError_t events_sample(const SweepPlan &p, const void *pts, cudaStream_t st)
 {
     const int n = p.n;
-    { StageTimer _t(STAGE_SAMPLE, st); k_sample<G><<<(p.S + 255) / 256, 256, 0, st>>>(pts, n, p.emax, p.S, p.skeys); }
-    const long long *src = sort_sample(p.skeys, p.skeys2, p.S, st);
+    { StageTimer _t(STAGE_SAMPLE, st); k_sample<G><<<(p.S + 255) / 256, 256, 0, st>>>(p.skip, pts, n, p.emax, p.S, p.skeys); }
+    const long long *src = sort_sample(p.skip, p.skeys, p.skeys2, p.S, st);
     {
         const size_t qs = (size_t)BND_MAX / 2 * 8;
         cudaFuncSetAttribute(k_splitters, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)qs);
         StageTimer _t(STAGE_SPLITTERS, st);
-        k_splitters<<<1, 1024, qs, st>>>(src, p.S, p.B, p.bnd, p.meta);
+        k_splitters<<<1, 1024, qs, st>>>(p.skip, src, p.S, p.B, p.bnd, p.meta);
     }
     return cudaGetLastError();
 }
@@ -2573,11 +2584,11 @@ static cudaError_t events_count(const SweepPlan &p, const void *pts, cudaStream_
     {
         cudaFuncSetAttribute(k_bucket_pairs<false, G>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cnt_smem);
         StageTimer _t(STAGE_COUNT_PAIRS, st);
-        k_bucket_pairs<false, G><<<p.C, CNT_THREADS, cnt_smem, st>>>(pts, p.n, p.bnd, p.meta, p.hist, nullptr, nullptr,
+        k_bucket_pairs<false, G><<<p.C, CNT_THREADS, cnt_smem, st>>>(p.skip, pts, p.n, p.bnd, p.meta, p.hist, nullptr, nullptr,
                                                                     nullptr);
     }
-    { StageTimer _t(STAGE_PREFIX, st); k_bucket_prefix<<<(BND_MAX + 255) / 256, 256, 0, st>>>(p.hist, p.C, p.meta, p.base); }
-    { StageTimer _t(STAGE_SCAN, st); k_bucket_scan<<<1, 1024, 0, st>>>(p.base, p.meta); }
+    { StageTimer _t(STAGE_PREFIX, st); k_bucket_prefix<<<(BND_MAX + 255) / 256, 256, 0, st>>>(p.skip, p.hist, p.C, p.meta, p.base); }
+    { StageTimer _t(STAGE_SCAN, st); k_bucket_scan<<<1, 1024, 0, st>>>(p.skip, p.base, p.meta); }
     return cudaGetLastError();
 }
 
@@ -2635,9 +2646,9 @@ cudaError_t launch_sweep_count(const SweepPlan &p, const unsigned char *keep, co
         StageTimer _t(STAGE_OTHER, st);
         k_distinct_x_pairs<<<1, 1024, 32768 * 4, st>>>(p.xy, n, p.meta);
     }
-    { StageTimer _t(STAGE_PREFIX, st); k_bucket_prefix<<<(BND_MAX + 255) / 256, 256, 0, st>>>(p.hist, p.C, p.meta, p.base); }
+    { StageTimer _t(STAGE_PREFIX, st); k_bucket_prefix<<<(BND_MAX + 255) / 256, 256, 0, st>>>(p.skip, p.hist, p.C, p.meta, p.base); }
     // without a resplit the list scatter's cursors are these bucket starts
-    { StageTimer _t(STAGE_SCAN, st); k_bucket_scan<<<1, 1024, 0, st>>>(p.base, p.meta, p.resplit ? nullptr : p.hist); }
+    { StageTimer _t(STAGE_SCAN, st); k_bucket_scan<<<1, 1024, 0, st>>>(p.skip, p.base, p.meta, p.resplit ? nullptr : p.hist); }
     return cudaGetLastError();
 }
 
@@ -2666,17 +2677,17 @@ cudaError_t launch_events_finish(const SweepPlan &p, const void *pts, const unsi
         if (p.resplit) {
             const int S2 = std::min(p.S, RESPLIT_S);
             { StageTimer _t(STAGE_SAMPLE, st); k_list_sample<G><<<(S2 + 255) / 256, 256, 0, st>>>(pts, p.ev2, p.meta + 6, S2, p.skeys); }
-            const long long *src = sort_sample(p.skeys, p.skeys2, S2, st);
+            const long long *src = sort_sample(p.skip, p.skeys, p.skeys2, S2, st);
             {
                 StageTimer _t(STAGE_SPLITTERS, st);
                 const size_t qs = (size_t)BND_MAX / 2 * 8;
                 cudaFuncSetAttribute(k_splitters, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)qs);
-                k_splitters<<<1, 1024, qs, st>>>(src, S2, BND_MAX / 2, p.bnd2, p.meta2, p.meta + 6, RESPLIT_PER);
+                k_splitters<<<1, 1024, qs, st>>>(p.skip, src, S2, BND_MAX / 2, p.bnd2, p.meta2, p.meta + 6, RESPLIT_PER);
             }
             if (cudaMemsetAsync(p.base2, 0, (size_t)(BND_MAX + 1) * 4, st) != cudaSuccess) return cudaGetLastError();
             cudaFuncSetAttribute(k_list_hist<G>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bsm);
             { StageTimer _t(STAGE_COUNT_PAIRS, st); k_list_hist<G><<<p.C, CNT_THREADS, bsm, st>>>(pts, p.bnd2, p.meta2, p.ev2, p.meta + 6, p.base2); }
-            { StageTimer _t(STAGE_SCAN, st); k_bucket_scan<<<1, 1024, 0, st>>>(p.base2, p.meta2, cursor); }
+            { StageTimer _t(STAGE_SCAN, st); k_bucket_scan<<<1, 1024, 0, st>>>(p.skip, p.base2, p.meta2, cursor); }
             sbnd = p.bnd2;
             sbase = p.base2;
             smeta = p.meta2;
@@ -2687,24 +2698,24 @@ cudaError_t launch_events_finish(const SweepPlan &p, const void *pts, const unsi
         k_scatter_list<G><<<p.C, CNT_THREADS, bsm, st>>>(pts, sbnd, smeta, p.ev2, cursor, p.ev, p.meta + 6);
     } else {
         StageTimer _t(STAGE_SCATTER, st);
-        k_bucket_pairs<true, G><<<p.C, CNT_THREADS, cnt_smem, st>>>(pts, n, p.bnd, p.meta, p.hist, p.base, p.ev, keep);
+        k_bucket_pairs<true, G><<<p.C, CNT_THREADS, cnt_smem, st>>>(p.skip, pts, n, p.bnd, p.meta, p.hist, p.base, p.ev, keep);
     }
     const size_t seg_smem = (size_t)SEG_CAP * 12;
     cudaFuncSetAttribute(k_segsort<G>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)seg_smem);
-    { StageTimer _t(STAGE_SEGSORT, st); k_segsort<G><<<p.C, 1024, seg_smem, st>>>(pts, p.ev, sbase, sbnd, smeta, p.oversize); }
+    { StageTimer _t(STAGE_SEGSORT, st); k_segsort<G><<<p.C, 1024, seg_smem, st>>>(p.skip, pts, p.ev, sbase, sbnd, smeta, p.oversize); }
     if (p.emax > SEG_CAP) {
         cudaFuncSetAttribute(k_segsort_big<G>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)seg_smem);
         StageTimer _t(STAGE_SEGSORT_BIG, st);
-        k_segsort_big<G><<<p.C, 1024, seg_smem, st>>>(pts, p.ev, p.ev2, sbase, smeta, p.oversize);
+        k_segsort_big<G><<<p.C, 1024, seg_smem, st>>>(p.skip, pts, p.ev, p.ev2, sbase, smeta, p.oversize);
     }
     {
         StageTimer _t(STAGE_PLAN, st);
-        if (plan) k_plan<<<(p.W + 7) / 8, 256, 0, st>>>(p.ev, p.base, p.meta, p.W, p.range);
+        if (plan) k_plan<<<(p.W + 7) / 8, 256, 0, st>>>(p.skip, p.ev, p.base, p.meta, p.W, p.range);
         else k_snap_ranges<<<(2 * p.W + 7) / 8, 256, 0, st>>>(p.ev, p.base, p.meta, 2 * p.W, p.range);
     }
     {
         StageTimer _t(STAGE_PLAN, st);
-        k_monotone_ranges<<<1, 1024, 0, st>>>(p.range, 2 * p.W);
+        k_monotone_ranges<<<1, 1024, 0, st>>>(p.skip, p.range, 2 * p.W);
     }
     return cudaGetLastError();
 }

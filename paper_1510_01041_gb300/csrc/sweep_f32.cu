@@ -107,9 +107,10 @@ __device__ __forceinline__ bool tame(float v)
 
 // One CTA: pack the coordinates, record whether all of them are finite
 // (bad[0]) and whether all of them are tame (bad[1]).
-__global__ void __launch_bounds__(1024) k_pack_f32(const float *__restrict__ x, const float *__restrict__ y, int n,
+__global__ void __launch_bounds__(1024) k_pack_f32(const int *skip, const float *__restrict__ x, const float *__restrict__ y, int n,
                                                    float2 *__restrict__ P, int *__restrict__ bad)
 {
+    if (skip && *skip) return;
     int nf = 0, wild = 0;
     for (int k = threadIdx.x; k < n; k += blockDim.x) {
         const float2 v = make_float2(x[k], y[k]);
@@ -127,7 +128,7 @@ __global__ void __launch_bounds__(1024) k_pack_f32(const float *__restrict__ x, 
 
 // Sweeper start: sort by (z at the first slope, x ascending, index), score
 // every window.  keys/idx: shared memory (n <= 8192) or global scratch.
-__global__ void __launch_bounds__(1024) k_sweep_init_f32(const float2 *__restrict__ P, int n, int h,
+__global__ void __launch_bounds__(1024) k_sweep_init_f32(const int *skip, const float2 *__restrict__ P, int n, int h,
                                                          const unsigned *__restrict__ ev,
                                                          const unsigned *__restrict__ range, int W,
                                                          int *__restrict__ meta_mut,
@@ -136,6 +137,7 @@ __global__ void __launch_bounds__(1024) k_sweep_init_f32(const float2 *__restric
                                                          long long *__restrict__ gkeys, unsigned short *__restrict__ gidx,
                                                          CandF *__restrict__ cands)
 {
+    if (skip && *skip) return;
     const int *meta = meta_mut;
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ double s_slope;
@@ -277,13 +279,14 @@ __device__ __forceinline__ bool f32_wider(float2 A, float2 T, float sf, bool top
 // batch); a pair that is not adjacent is repaired by the whole warp.  Each
 // swap scores its two windows, the float pre-test first.
 template <bool XY_SMEM>
-__global__ void __launch_bounds__(256) k_sweep_f32(const float2 *__restrict__ g_p, int n, int h,
+__global__ void __launch_bounds__(256) k_sweep_f32(const int *skip, const float2 *__restrict__ g_p, int n, int h,
                                                    const unsigned *__restrict__ ev,
                                                    const unsigned *__restrict__ range, int W,
                                                    const unsigned short *__restrict__ orders,
                                                    CandF *__restrict__ cands, int *__restrict__ meta,
                                                    const int *__restrict__ flags)
 {
+    if (skip && *skip) return;
     extern __shared__ __align__(16) unsigned char smem[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
     unsigned *next_range = reinterpret_cast<unsigned *>(meta + 4);
@@ -469,9 +472,10 @@ __global__ void __launch_bounds__(256) k_sweep_f32(const float2 *__restrict__ g_
     if (lane == 0) cands[W + g] = best;
 }
 
-__global__ void __launch_bounds__(1024) k_argmin_f32(const CandF *__restrict__ cands, int count,
+__global__ void __launch_bounds__(1024) k_argmin_f32(const int *skip, const CandF *__restrict__ cands, int count,
                                                      const int *__restrict__ bad, lms_result *__restrict__ out)
 {
+    if (skip && *skip) return;
     __shared__ CandF s_best[32];
     CandF best = candf_empty();
     for (int k = threadIdx.x; k < count; k += blockDim.x)
@@ -535,7 +539,7 @@ cudaError_t launch_sweep_f32_fit(const SweepPlan &p, const float *x, const float
         q += a256((size_t)p.W * Pn * 8);
         gidx = reinterpret_cast<unsigned short *>(q);
     }
-    { StageTimer _t(STAGE_PACK, st); k_pack_f32<<<1, 1024, 0, st>>>(x, y, n, P, bad); }
+    { StageTimer _t(STAGE_PACK, st); k_pack_f32<<<1, 1024, 0, st>>>(p.skip, x, y, n, P, bad); }
     cudaError_t e = launch_events_prepare<KeyF32>(p, P, st);
     if (e != cudaSuccess) return e;
     e = launch_events_finish<KeyF32>(p, P, nullptr, st, true);
@@ -545,7 +549,7 @@ cudaError_t launch_sweep_f32_fit(const SweepPlan &p, const float *x, const float
     cudaFuncSetAttribute(k_sweep_init_f32, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)init_smem);
     {
         StageTimer _t(STAGE_INIT, st);
-        k_sweep_init_f32<<<p.W, 1024, init_smem, st>>>(P, n, p.h, p.ev, p.range, p.W, p.meta, p.base, p.orders, gkeys,
+        k_sweep_init_f32<<<p.W, 1024, init_smem, st>>>(p.skip, P, n, p.h, p.ev, p.range, p.W, p.meta, p.base, p.orders, gkeys,
                                                       gidx, cands);
     }
     const size_t per = 2 * (((size_t)n * 2 + 15) / 16 * 16);
@@ -561,17 +565,17 @@ cudaError_t launch_sweep_f32_fit(const SweepPlan &p, const float *x, const float
     if (xs) {
         cudaFuncSetAttribute(k_sweep_f32<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sw_smem);
         StageTimer _t(STAGE_SWEEP, st);
-        k_sweep_f32<true><<<blocks, 32 * spb, sw_smem, st>>>(P, n, p.h, p.ev, p.range, p.W, p.orders, cands, p.meta,
+        k_sweep_f32<true><<<blocks, 32 * spb, sw_smem, st>>>(p.skip, P, n, p.h, p.ev, p.range, p.W, p.orders, cands, p.meta,
                                                              bad);
     } else {
         cudaFuncSetAttribute(k_sweep_f32<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sw_smem);
         StageTimer _t(STAGE_SWEEP, st);
-        k_sweep_f32<false><<<blocks, 32 * spb, sw_smem, st>>>(P, n, p.h, p.ev, p.range, p.W, p.orders, cands, p.meta,
+        k_sweep_f32<false><<<blocks, 32 * spb, sw_smem, st>>>(p.skip, P, n, p.h, p.ev, p.range, p.W, p.orders, cands, p.meta,
                                                               bad);
     }
     {
         StageTimer _t(STAGE_ARGMIN, st);
-        k_argmin_f32<<<1, 1024, 0, st>>>(cands, p.W + G, bad, out);
+        k_argmin_f32<<<1, 1024, 0, st>>>(p.skip, cands, p.W + G, bad, out);
     }
     return cudaGetLastError();
 }

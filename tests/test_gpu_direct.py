@@ -90,3 +90,23 @@ def test_batch_equals_sweep(L):
         want = L.decode(L.fit(X[a:b], Y[a:b], int(h[k]), "sweep"))[0]
         assert tuple(r[f] for f in F) == tuple(want[f] for f in F), (k, b - a, r, want)
         assert r["algorithm"] == L.ALGOS["bnb" if b - a >= 512 else "sweep"]
+
+
+@pytest.mark.parametrize("n", [15, 16, 17, 64, 511, 2048, 2049, 4096, 4097])
+def test_float_equals_sweep(L, n):
+    """The float form (grid points, scores in double) finds the sweep's line: the same pair, and a width that
+    differs by the rounding of double projections only (2^-53 of their size, at most 1e-9 of the width here)."""
+    rng = np.random.default_rng(n)
+    cases = [datagen.gaussian_f32(n, n, f) for f in (0.4, 0.0, 1.0)]
+    cases += [(rng.standard_cauchy(n), rng.standard_cauchy(n)), (np.full(n, 3.0), rng.normal(size=n)),
+              (3 + 1e-6 * rng.normal(size=n), rng.normal(size=n)),
+              (rng.normal(size=n) * 1e-9, rng.normal(size=n) * 1e9),
+              (np.append(rng.normal(size=n - 1), np.inf), rng.normal(size=n))]
+    for k, (x, y) in enumerate(cases):
+        X, Y = (torch.from_numpy(np.ascontiguousarray(a, dtype=np.float32)).cuda() for a in (x, y))
+        for h in (0, int(0.75 * n)):
+            a, b = L.decode(L.fit(X, Y, h))[0], L.decode(L.fit(X, Y, h, "sweep"))[0]
+            assert a["status"] == b["status"] and a["algorithm"] == b["algorithm"], (k, n, h, a, b)
+            if a["status"] == 0:
+                assert (a["i"], a["j"], a["theta1"]) == (b["i"], b["j"], b["theta1"]), (k, n, h, a, b)
+                assert a["med_sq"] == pytest.approx(b["med_sq"], rel=1e-9), (k, n, h, a, b)
