@@ -71,7 +71,8 @@ enum lms_dtype {
 };
 
 enum lms_algo {
-    LMS_ALGO_AUTO = 0,        /* library choice */
+    LMS_ALGO_AUTO = 0,        /* library choice; reports PLAIN (int16 up to 512 points) or SWEEP, whose record it
+                                 equals, also where a branch-and-bound drops slopes that cannot win */
     LMS_ALGO_PLAIN = 1,       /* sort the projections at every pairwise slope (n <= 1024) */
     LMS_ALGO_SWEEP = 2,       /* exact kinetic sweep over slope-sorted events */
     LMS_ALGO_BNB = 3,         /* seeded branch-and-bound over slope intervals + sweep of survivors */
@@ -222,7 +223,8 @@ LMS_API int lms_fit_learned_host(lms_setnet *net, const void *x, const void *y, 
  * lms_batch_plan_create sizes everything from the host offsets once: sets
  * with at most plain_max_n points (0 = 256, at most 256) go to one
  * persistent plain kernel over (set, run of slopes) work items in three
- * size classes; larger sets (up to 32768 points) each get the exact sweep
+ * size classes (up to 64 points; above, to one CTA of the one-kernel
+ * branch-and-bound, with the same record); larger sets (up to 32768 points) each get the exact sweep
  * of every slope or, from 512 points on, the exact branch-and-bound, spread
  * over `streams` internal streams (0 = 8).  It allocates the plan's
  * device memory and waits for the device.
