@@ -82,8 +82,8 @@ struct Choice {
     int plain_warps;
     int sms;
     bool direct;      // by the one-kernel branch-and-bound (direct.cu), reported as `algo`
-    size_t direct_bytes;
-    size_t bytes;
+    size_t bytes;     // the same for every route of one n, dtype and options: a fit by one route never
+                      // moves the workspace that a captured fit by another one uses
     size_t bnb_off;   // offset of the branch-and-bound scratch
     size_t f32_off;   // offset of the float32 sweep scratch
 };
@@ -114,7 +114,6 @@ int choose(int n, int h, int dtype, const lms_options *opt, int dev, Choice &c)
     // (up to 512 points the per-slope kernel is as fast: 0.05 / 0.30 ms at 256 /
     // 509 points against 0.27 / 0.20 - 0.35 ms)
     c.direct = algo_req == LMS_ALGO_AUTO && algo == LMS_ALGO_SWEEP && dtype == LMS_I16 && direct_ok(n, h);
-    c.direct_bytes = c.direct ? direct_bytes(n) + 256 : 0;   // 256: result staging for host-pointer calls
     if (algo == LMS_ALGO_PLAIN) {
         if (n > 1024) return LMS_ERR_UNSUPPORTED;
         c.plain_warps = plain_warps_for(n, sms);
@@ -138,10 +137,9 @@ int choose(int n, int h, int dtype, const lms_options *opt, int dev, Choice &c)
         return LMS_ERR_ARG;
     }
     c.bytes += 256;   // result staging for host-pointer calls, and the flag of a float fit
-    if (dtype == LMS_F32 && algo_req == LMS_ALGO_AUTO && direct_f32_ok(n, h) && direct_f32_bytes(n) + 256 <= c.bytes) {
-        c.direct = true;
-        c.direct_bytes = c.bytes;
-    }
+    if (dtype == LMS_F32) c.direct = algo_req == LMS_ALGO_AUTO && direct_f32_ok(n, h);
+    // the one kernel's scratch lies in the same workspace (it needs far less: 2.8 MB of 42 at n = 2048)
+    if (c.direct && (dtype == LMS_F32 ? direct_f32_bytes(n) : direct_bytes(n)) + 256 > c.bytes) c.direct = false;
     return LMS_OK;
 }
 
@@ -240,12 +238,16 @@ int fit_bnb_after(const void *x, const void *y, int64_t n, int64_t h, const floa
     if (rc) return rc;
     int dev;
     if (current_device(dev)) return LMS_ERR_CUDA;
+    Choice c;
+    rc = choose((int)n, (int)h, LMS_I16, &o, dev, c);
+    if (rc) return rc;
     void *ws = nullptr;
+    rc = workspace(c.bytes, st, &ws);
+    if (rc) return rc;
     // the statistics, the seed modes and the sweep's tuning options belong to
     // the staged branch-and-bound; without them one kernel does it all
-    if (!stats && o.seed_mode == 0 && o.sweepers == 0 && o.buckets == 0 && direct_ok((int)n, (int)h)) {
-        rc = workspace(direct_bytes((int)n), st, &ws);
-        if (rc) return rc;
+    if (!stats && o.seed_mode == 0 && o.sweepers == 0 && o.buckets == 0 && direct_ok((int)n, (int)h) &&
+        direct_bytes((int)n) <= c.bytes) {
         if (pred_ready && cudaStreamWaitEvent(st, pred_ready, 0) != cudaSuccess) return LMS_ERR_CUDA;
         cudaGetLastError();
         return launch_direct((const short *)x, (const short *)y, (int)n, (int)h, LMS_ALGO_BNB, seed_slope, out, ws,
@@ -253,11 +255,6 @@ int fit_bnb_after(const void *x, const void *y, int64_t n, int64_t h, const floa
                    ? LMS_OK
                    : LMS_ERR_CUDA;
     }
-    Choice c;
-    rc = choose((int)n, (int)h, LMS_I16, &o, dev, c);
-    if (rc) return rc;
-    rc = workspace(c.bytes, st, &ws);
-    if (rc) return rc;
     SweepPlan p = c.sweep;
     sweep_plan_carve(p, ws);
     cudaGetLastError();
@@ -283,7 +280,7 @@ int lms_fit(const void *x, const void *y, int64_t n, int64_t h, int32_t dtype, c
     if (rc) return rc;
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
     void *ws = nullptr;
-    rc = workspace(c.direct ? c.direct_bytes : c.bytes, st, &ws);
+    rc = workspace(c.bytes, st, &ws);
     if (rc) return rc;
     return run_fit(x, y, (int)n, (int)h, dtype, opt, out, st, ws, c);
 }
@@ -302,13 +299,12 @@ int lms_fit_host(const void *x, const void *y, int64_t n, int64_t h, int32_t dty
     const size_t in_bytes = ((size_t)n * esz + 255) / 256 * 256;
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
     void *ws = nullptr;
-    const size_t fit_bytes = c.direct ? c.direct_bytes : c.bytes;   // below c.bytes, so any workspace sized for it will do
-    rc = workspace(fit_bytes + 2 * in_bytes, st, &ws);
+    rc = workspace(c.bytes + 2 * in_bytes, st, &ws);
     if (rc) return rc;
     unsigned char *base = static_cast<unsigned char *>(ws);
-    unsigned char *dx = base + fit_bytes;
+    unsigned char *dx = base + c.bytes;
     unsigned char *dy = dx + in_bytes;
-    lms_result *dres = reinterpret_cast<lms_result *>(base + fit_bytes - 256);
+    lms_result *dres = reinterpret_cast<lms_result *>(base + c.bytes - 256);
     if (cudaMemcpyAsync(dx, x, (size_t)n * esz, cudaMemcpyHostToDevice, st) != cudaSuccess) return LMS_ERR_CUDA;
     if (cudaMemcpyAsync(dy, y, (size_t)n * esz, cudaMemcpyHostToDevice, st) != cudaSuccess) return LMS_ERR_CUDA;
     rc = run_fit(dx, dy, (int)n, (int)h, dtype, opt, dres, st, ws, c);

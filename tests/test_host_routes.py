@@ -1,0 +1,58 @@
+"""Host routes without a GPU: workspaces, launches and error returns of the
+library's own host code over the stand-in runtime (host_library.py)."""
+import ctypes
+
+import pytest
+
+import host_library
+
+I16, F32 = 0, 1
+
+
+@pytest.fixture()
+def H(tmp_path):
+    return host_library.load(tmp_path)
+
+
+# ---------------------------------------------------------------- workspaces
+@pytest.mark.parametrize("n", [64, 513, 2048, 4096, 8192, 16385, 65536])
+def test_every_route_of_one_size_uses_one_workspace(H, n):
+    """A fit captured in a graph keeps the workspace's address: later fits of the same n by another route (with
+    statistics, an order statistic below n / 8) neither move nor free the buffer, and all of them fit in it while
+    streams are being captured."""
+    assert H.fit_bnb(n) == 0
+    frees, held = H.lib.fake_frees(), H.lib.fake_held()
+    H.set("capturing", 1)
+    assert H.fit_bnb(n, h=max(1, n // 16)) == 0
+    assert H.fit_bnb(n, stats=True) == 0
+    assert H.fit_bnb(n) == 0
+    assert (H.lib.fake_frees(), H.lib.fake_held()) == (frees, held)
+
+
+@pytest.mark.parametrize("n,dtype", [(513, I16), (2048, I16), (8192, I16), (16385, I16), (64, F32), (2048, F32),
+                                     (4096, F32)])
+def test_auto_and_sweep_use_one_workspace(H, n, dtype):
+    assert H.fit(n, dtype=dtype) == 0
+    frees = H.lib.fake_frees()
+    H.set("capturing", 1)
+    for h in (0, max(1, n // 16)):
+        assert H.fit(n, h, dtype=dtype) == 0
+        assert H.fit(n, h, "sweep", dtype=dtype) == 0
+    assert H.lib.fake_frees() == frees
+
+
+@pytest.mark.parametrize("n,dtype,algorithm", [(600, I16, "auto"), (8192, I16, "auto"), (64, I16, "bnb"),
+                                               (8192, I16, "bnb"), (2048, F32, "auto")])
+def test_installed_workspace(H, n, dtype, algorithm):
+    """lms_workspace_size bytes are enough for every route; less than the fit's share of them is refused by all."""
+    size = H.workspace_size(n, dtype, algorithm)
+    staging = 2 * ((n * (4 if dtype == F32 else 2) + 255) // 256 * 256)
+    buf = ctypes.create_string_buffer(size)
+    runs = [lambda: H.fit(n, 0, algorithm, dtype), lambda: H.fit(n, 1, algorithm, dtype)]
+    if algorithm == "bnb":
+        runs += [lambda: H.fit_bnb(n), lambda: H.fit_bnb(n, stats=True)]
+    H.set_workspace(buf, size)
+    assert H.fit(n, 0, algorithm, dtype, host=True) == 0
+    assert [r() for r in runs] == [0] * len(runs)
+    H.set_workspace(buf, size - staging - 1)
+    assert [r() for r in runs] == [6] * len(runs)   # LMS_ERR_WORKSPACE
