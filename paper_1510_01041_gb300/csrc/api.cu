@@ -5,8 +5,10 @@
 // host only enqueues work on the caller's stream.
 #include <cuda_runtime.h>
 
+#include <map>
 #include <mutex>
 #include <string.h>
+#include <utility>
 
 #include "common.cuh"
 #include "kernels.cuh"
@@ -213,6 +215,20 @@ int run_fit(const void *x, const void *y, int n, int h, int dtype, const lms_opt
 }
 
 }  // namespace
+
+cudaError_t allow_smem_of(const void *kernel, size_t bytes)
+{
+    static std::mutex mu;
+    static std::map<std::pair<int, const void *>, size_t> limits;
+    int dev;
+    if (current_device(dev)) return cudaErrorInvalidDevice;
+    std::lock_guard<std::mutex> lock(mu);
+    size_t &limit = limits.try_emplace({dev, kernel}, (size_t)48 * 1024).first->second;
+    if (bytes <= limit) return cudaSuccess;
+    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    if (e == cudaSuccess) limit = bytes;
+    return e;
+}
 
 unsigned long long workspace_generation()
 {

@@ -1209,7 +1209,7 @@ int run_bnb(const SweepPlan &p, const short *x, const short *y, const float *pre
     if (launch_sample_counts(p, scount, st) != cudaSuccess) return LMS_ERR_CUDA;
     {
         StageTimer _t(STAGE_SEEDS, st);
-        cudaFuncSetAttribute(k_x_center, cudaFuncAttributeMaxDynamicSharedMemorySize, 32768 * 4);
+        allow_smem(k_x_center, 32768 * 4);
         k_x_center<<<1, 1024, 32768 * 4, st>>>(p.xy, n, h, xc);
     }
     if (pred_ready && cudaStreamWaitEvent(st, pred_ready, 0) != cudaSuccess) return LMS_ERR_CUDA;
@@ -1221,8 +1221,8 @@ int run_bnb(const SweepPlan &p, const short *x, const short *y, const float *pre
     // 32-bit keys: one sorted array plus merge scratch; two sorted arrays plus scratch
     const size_t one_sort = (n <= BNB_SMEM_N) ? (size_t)2 * Ps * 4 : (size_t)2 * BNB_SMEM_N * 4;
     const size_t two_sorts = (n <= BNB_SMEM_N) ? (size_t)3 * Ps * 4 : (size_t)2 * BNB_SMEM_N * 4;
-    cudaFuncSetAttribute(k_score_dyadic, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)one_sort);
-    cudaFuncSetAttribute(k_node_lb, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)two_sorts);
+    allow_smem(k_score_dyadic, one_sort);
+    allow_smem(k_node_lb, two_sorts);
     {
         StageTimer _t(STAGE_SEEDS, st);
         k_score_dyadic<<<std::min(KS, grid), 1024, one_sort, st>>>(p.xy, n, h, xc, seed_keys, KS, seed_w, gscr);
@@ -1241,8 +1241,8 @@ int run_bnb(const SweepPlan &p, const short *x, const short *y, const float *pre
     }
     // the interval tree, level by level, all on the device
     const size_t tree_smem = (size_t)(BND_MAX + 1) * sizeof(unsigned);
-    cudaFuncSetAttribute(k_tree_first, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tree_smem);
-    cudaFuncSetAttribute(k_tree_step, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tree_smem);
+    allow_smem(k_tree_first, tree_smem);
+    allow_smem(k_tree_step, tree_smem);
     {
         StageTimer _t(STAGE_TREE, st);
         k_tree_first<<<1, TREE_THREADS, tree_smem, st>>>(scount, p.meta, p.bnd, sms, sbase, nodes[0], nkeys[0], keep,

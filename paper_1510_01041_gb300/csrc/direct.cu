@@ -2332,7 +2332,7 @@ cudaError_t launch_cluster(const DirectArgs &a, size_t smem, cudaStream_t st)
 {
     auto kern = SH::kernel;
     const int C = a.shape.C;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(kern, smem);
     if (e == cudaSuccess && C > 8) e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
@@ -2419,7 +2419,7 @@ int direct_batch_teams(int nsets, int nmax, int sms)
 {
     auto kern = Batch::kernel;
     const size_t smem = Batch::smem(nmax, batch_shape(nmax).HC);
-    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    allow_smem(kern, smem);
     int occ = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, Batch::T, smem) != cudaSuccess || occ < 1) {
         cudaGetLastError();
@@ -2455,7 +2455,7 @@ cudaError_t launch_direct_batch(const short *x, const short *y, const long long 
     cudaError_t e = cudaMemsetAsync(a.next, 0, sizeof(int), st);
     if (e != cudaSuccess) return e;
     auto kern = Batch::kernel;
-    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    e = allow_smem(kern, smem);
     if (e != cudaSuccess) return e;
     StageTimer _t(STAGE_DIRECT, st);
     kern<<<nteams, Batch::T, smem, st>>>(a);

@@ -498,12 +498,12 @@ int lms_hough_refine(const uint8_t *edges, int64_t B, int32_t H, int32_t W, int3
     }
     const size_t vsm = sizeof(int) * TT * (size_t)n_rho;
     if (vsm > 227 * 1024) { cudaFree(mem); return LMS_ERR_UNSUPPORTED; }
-    cudaFuncSetAttribute(k_vote, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)vsm);
+    allow_smem(k_vote, vsm);
     {
         StageTimer _t(STAGE_HOUGH, st);
         k_vote<<<dim3((n_theta + TT - 1) / TT, (unsigned)B), 1024, vsm, st>>>(pts, img_off, cs, n_theta, n_rho, acc);
     }
-    cudaFuncSetAttribute(k_peaks, cudaFuncAttributeMaxDynamicSharedMemorySize, PEAK_SMEM * 8);
+    allow_smem(k_peaks, PEAK_SMEM * 8);
     {
         StageTimer _t(STAGE_HOUGH, st);
         k_peaks<<<(unsigned)B, 1024, PEAK_SMEM * 8, st>>>(acc, n_theta, n_rho, top_k, nms_theta, nms_rho, peaks, gcand,
@@ -540,7 +540,7 @@ int lms_hough_refine(const uint8_t *edges, int64_t B, int32_t H, int32_t W, int3
         k_gather<true><<<dim3(64, (unsigned)B), 256, 0, st>>>(pts, img_off, cs, n_rho, peaks, top_k, band_px, scnt,
                                                              soff, keys);
     }
-    cudaFuncSetAttribute(k_set_finish, cudaFuncAttributeMaxDynamicSharedMemorySize, 32768 * 4);
+    allow_smem(k_set_finish, 32768 * 4);
     {
         StageTimer _t(STAGE_HOUGH, st);
         k_set_finish<<<(unsigned)(B * top_k), 1024, 32768 * 4, st>>>(pts, img_off, cs, peaks, top_k, soff, keys, sx,

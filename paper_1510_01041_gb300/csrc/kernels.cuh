@@ -31,6 +31,18 @@ class StageTimer {
     cudaEvent_t a_;
 };
 
+// Lets `kernel` be launched with `bytes` of dynamic shared memory on the
+// current device.  The limit belongs to the kernel, not to the call: host
+// threads that launch the same kernel at other sizes share it, so it is only
+// ever raised (a lower limit set between another thread's call and its launch
+// would refuse that launch).
+cudaError_t allow_smem_of(const void *kernel, size_t bytes);
+template <class F>
+cudaError_t allow_smem(F *kernel, size_t bytes)
+{
+    return allow_smem_of(reinterpret_cast<const void *>(kernel), bytes);
+}
+
 // Slope-key policies for the event pipeline: key() returns false when the
 // pair has no slope (equal x) and otherwise an int64 key that orders slopes.
 struct KeyI16 {   // packed int16 points: exact key floor(dy 2^32 / dx)

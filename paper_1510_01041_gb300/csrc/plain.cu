@@ -197,7 +197,7 @@ cudaError_t launch_plain(const short *x, const short *y, int n, int h, Cand *can
     const long long npairs = (long long)n * (n - 1) / 2;
 #define LMS_PLAIN_CASE(EE)                                                                     \
     case EE:                                                                                   \
-        cudaFuncSetAttribute(k_plain<EE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem); \
+        allow_smem(k_plain<EE>, smem);                                                         \
         { StageTimer _t(STAGE_PLAIN, st);                                                      \
         k_plain<EE><<<blocks, threads, smem, st>>>(x, y, n, h, npairs, cands); }                \
         break;

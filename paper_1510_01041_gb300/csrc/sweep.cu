@@ -2452,10 +2452,10 @@ void sweep_plan_configure(SweepPlan &p, int n, int h, int sms, int want_w, int w
     const size_t sw_smem = sweep_smem_bytes(n, p.xy_smem, p.pos_smem, spb);
     int per_sm = 0;
     if (p.xy_smem) {
-        cudaFuncSetAttribute(k_sweep<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sw_smem);
+        allow_smem(k_sweep<true>, sw_smem);
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sweep<true>, 32 * spb, sw_smem);
     } else {
-        cudaFuncSetAttribute(k_sweep<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sw_smem);
+        allow_smem(k_sweep<false>, sw_smem);
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sweep<false>, 32 * spb, sw_smem);
     }
     cudaGetLastError();
@@ -2555,7 +2555,7 @@ static long long *sort_sample(const int *skip, long long *keys, long long *scrat
 {
     const int P = std::min(S, SAMPLE_CH);
     const size_t smem = (size_t)2 * P * 8;
-    cudaFuncSetAttribute(k_sort_chunks, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    allow_smem(k_sort_chunks, smem);
     { StageTimer _t(STAGE_SAMPLE_SORT, st); k_sort_chunks<<<S / P, 1024, smem, st>>>(skip, keys, S); }
     if (S <= SAMPLE_CH) return keys;
     { StageTimer _t(STAGE_SAMPLE_SORT, st); k_merge_chunks<<<(S + 255) / 256, 256, 0, st>>>(skip, keys, scratch, S); }
@@ -2570,7 +2570,7 @@ static cudaError_t events_sample(const SweepPlan &p, const void *pts, cudaStream
     const long long *src = sort_sample(p.skip, p.skeys, p.skeys2, p.S, st);
     {
         const size_t qs = (size_t)BND_MAX / 2 * 8;
-        cudaFuncSetAttribute(k_splitters, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)qs);
+        allow_smem(k_splitters, qs);
         StageTimer _t(STAGE_SPLITTERS, st);
         k_splitters<<<1, 1024, qs, st>>>(p.skip, src, p.S, p.B, p.bnd, p.meta);
     }
@@ -2582,7 +2582,7 @@ static cudaError_t events_count(const SweepPlan &p, const void *pts, cudaStream_
 {
     const size_t cnt_smem = (size_t)BND_MAX * 8 + (size_t)BND_MAX * 4;
     {
-        cudaFuncSetAttribute(k_bucket_pairs<false, G>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cnt_smem);
+        allow_smem(k_bucket_pairs<false, G>, cnt_smem);
         StageTimer _t(STAGE_COUNT_PAIRS, st);
         k_bucket_pairs<false, G><<<p.C, CNT_THREADS, cnt_smem, st>>>(p.skip, pts, p.n, p.bnd, p.meta, p.hist, nullptr, nullptr,
                                                                     nullptr);
@@ -2629,20 +2629,20 @@ cudaError_t launch_sweep_count(const SweepPlan &p, const unsigned char *keep, co
     unsigned long long *gscr = P > 8192 ? reinterpret_cast<unsigned long long *>(q) : nullptr;
     const size_t cnt_smem = (size_t)BND_MAX * 8 + (size_t)BND_MAX * 4;
     if (n <= TILE_COUNT_MAX_N) {
-        cudaFuncSetAttribute(k_tile_pairs, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cnt_smem);
+        allow_smem(k_tile_pairs, cnt_smem);
         StageTimer _t(STAGE_COUNT_PAIRS, st);
         k_tile_pairs<<<p.C, BAND_THREADS, cnt_smem, st>>>(p.xy, n, p.bnd, p.hist, keep, cov, p.meta, p.ev2);
     } else {
         const int Ps = P > 8192 ? 8192 : (P < 1024 ? 1024 : P);
         const size_t sort_smem = (size_t)2 * Ps * 8;
-        cudaFuncSetAttribute(k_band_sort, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sort_smem);
+        allow_smem(k_band_sort, sort_smem);
         { StageTimer _t(STAGE_COUNT_PAIRS, st); k_band_sort<<<PRE_MAX, 1024, sort_smem, st>>>(p.xy, n, cov, words, band, gscr); }
-        cudaFuncSetAttribute(k_band_pairs, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cnt_smem);
+        allow_smem(k_band_pairs, cnt_smem);
         StageTimer _t(STAGE_COUNT_PAIRS, st);
         k_band_pairs<<<p.C, BAND_THREADS, cnt_smem, st>>>(p.xy, n, p.bnd, p.hist, keep, cov, words, band, p.meta, p.ev2);
     }
     if (distinct_x) {
-        cudaFuncSetAttribute(k_distinct_x_pairs, cudaFuncAttributeMaxDynamicSharedMemorySize, 32768 * 4);
+        allow_smem(k_distinct_x_pairs, 32768 * 4);
         StageTimer _t(STAGE_OTHER, st);
         k_distinct_x_pairs<<<1, 1024, 32768 * 4, st>>>(p.xy, n, p.meta);
     }
@@ -2665,7 +2665,7 @@ cudaError_t launch_events_finish(const SweepPlan &p, const void *pts, const unsi
 {
     const int n = p.n;
     const size_t cnt_smem = (size_t)BND_MAX * 8 + (size_t)BND_MAX * 4;
-    cudaFuncSetAttribute(k_bucket_pairs<true, G>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cnt_smem);
+    allow_smem(k_bucket_pairs<true, G>, cnt_smem);
     // buckets of the bucket sorts: those of the count, or of a resplit
     const long long *sbnd = p.bnd;
     const unsigned *sbase = p.base;
@@ -2681,11 +2681,11 @@ cudaError_t launch_events_finish(const SweepPlan &p, const void *pts, const unsi
             {
                 StageTimer _t(STAGE_SPLITTERS, st);
                 const size_t qs = (size_t)BND_MAX / 2 * 8;
-                cudaFuncSetAttribute(k_splitters, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)qs);
+                allow_smem(k_splitters, qs);
                 k_splitters<<<1, 1024, qs, st>>>(p.skip, src, S2, BND_MAX / 2, p.bnd2, p.meta2, p.meta + 6, RESPLIT_PER);
             }
             if (cudaMemsetAsync(p.base2, 0, (size_t)(BND_MAX + 1) * 4, st) != cudaSuccess) return cudaGetLastError();
-            cudaFuncSetAttribute(k_list_hist<G>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bsm);
+            allow_smem(k_list_hist<G>, bsm);
             { StageTimer _t(STAGE_COUNT_PAIRS, st); k_list_hist<G><<<p.C, CNT_THREADS, bsm, st>>>(pts, p.bnd2, p.meta2, p.ev2, p.meta + 6, p.base2); }
             { StageTimer _t(STAGE_SCAN, st); k_bucket_scan<<<1, 1024, 0, st>>>(p.skip, p.base2, p.meta2, cursor); }
             sbnd = p.bnd2;
@@ -2693,7 +2693,7 @@ cudaError_t launch_events_finish(const SweepPlan &p, const void *pts, const unsi
             smeta = p.meta2;
         }
         // cursor: the bucket starts, written by the scan of the count (or of the resplit)
-        cudaFuncSetAttribute(k_scatter_list<G>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bsm);
+        allow_smem(k_scatter_list<G>, bsm);
         StageTimer _t(STAGE_SCATTER, st);
         k_scatter_list<G><<<p.C, CNT_THREADS, bsm, st>>>(pts, sbnd, smeta, p.ev2, cursor, p.ev, p.meta + 6);
     } else {
@@ -2701,10 +2701,10 @@ cudaError_t launch_events_finish(const SweepPlan &p, const void *pts, const unsi
         k_bucket_pairs<true, G><<<p.C, CNT_THREADS, cnt_smem, st>>>(p.skip, pts, n, p.bnd, p.meta, p.hist, p.base, p.ev, keep);
     }
     const size_t seg_smem = (size_t)SEG_CAP * 12;
-    cudaFuncSetAttribute(k_segsort<G>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)seg_smem);
+    allow_smem(k_segsort<G>, seg_smem);
     { StageTimer _t(STAGE_SEGSORT, st); k_segsort<G><<<p.C, 1024, seg_smem, st>>>(p.skip, pts, p.ev, sbase, sbnd, smeta, p.oversize); }
     if (p.emax > SEG_CAP) {
-        cudaFuncSetAttribute(k_segsort_big<G>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)seg_smem);
+        allow_smem(k_segsort_big<G>, seg_smem);
         StageTimer _t(STAGE_SEGSORT_BIG, st);
         k_segsort_big<G><<<p.C, 1024, seg_smem, st>>>(p.skip, pts, p.ev, p.ev2, sbase, smeta, p.oversize);
     }
@@ -2740,7 +2740,7 @@ cudaError_t launch_sweep_finish(const SweepPlan &p, const unsigned char *keep, c
     while (P < n) P <<= 1;
     // words + merge scratch (whole sort, or one 8192-word chunk above SORT_SMEM_N)
     const size_t init_smem = (n <= SORT_SMEM_N) ? (size_t)(P < 1024 ? 1024 : P) * 16 : (size_t)8192 * 16;
-    cudaFuncSetAttribute(k_sweep_init, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)init_smem);
+    allow_smem(k_sweep_init, init_smem);
     {
         StageTimer _t(STAGE_INIT, st);
         k_sweep_init<<<p.W, 1024, init_smem, st>>>(p.xy, n, p.h, p.ev, p.range, p.W, p.meta, p.base, p.orders,
@@ -2749,11 +2749,11 @@ cudaError_t launch_sweep_finish(const SweepPlan &p, const unsigned char *keep, c
     const size_t sw_smem = sweep_smem_bytes(n, p.xy_smem, p.pos_smem, p.spb);
     const int blocks = p.G / p.spb;
     if (p.xy_smem) {
-        cudaFuncSetAttribute(k_sweep<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sw_smem);
+        allow_smem(k_sweep<true>, sw_smem);
         StageTimer _t(STAGE_SWEEP, st);
         k_sweep<true><<<blocks, 32 * p.spb, sw_smem, st>>>(p.xy, n, p.h, p.ev, p.range, p.W, p.orders, p.cands, p.meta, p.gpos);
     } else {
-        cudaFuncSetAttribute(k_sweep<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sw_smem);
+        allow_smem(k_sweep<false>, sw_smem);
         StageTimer _t(STAGE_SWEEP, st);
         k_sweep<false><<<blocks, 32 * p.spb, sw_smem, st>>>(p.xy, n, p.h, p.ev, p.range, p.W, p.orders, p.cands, p.meta, p.gpos);
     }

@@ -546,7 +546,7 @@ cudaError_t launch_sweep_f32_fit(const SweepPlan &p, const float *x, const float
     if (e != cudaSuccess) return e;
     const int Ps = Pn < 1024 ? 1024 : Pn;
     const size_t init_smem = (n <= SORT_SMEM_N) ? (size_t)Ps * 16 : 0;   // sort words + merge scratch
-    cudaFuncSetAttribute(k_sweep_init_f32, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)init_smem);
+    allow_smem(k_sweep_init_f32, init_smem);
     {
         StageTimer _t(STAGE_INIT, st);
         k_sweep_init_f32<<<p.W, 1024, init_smem, st>>>(p.skip, P, n, p.h, p.ev, p.range, p.W, p.meta, p.base, p.orders, gkeys,
@@ -563,12 +563,12 @@ cudaError_t launch_sweep_f32_fit(const SweepPlan &p, const float *x, const float
     const int blocks = std::min((p.W + spb - 1) / spb, p.C);
     const int G = std::min(blocks * spb, p.W);
     if (xs) {
-        cudaFuncSetAttribute(k_sweep_f32<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sw_smem);
+        allow_smem(k_sweep_f32<true>, sw_smem);
         StageTimer _t(STAGE_SWEEP, st);
         k_sweep_f32<true><<<blocks, 32 * spb, sw_smem, st>>>(p.skip, P, n, p.h, p.ev, p.range, p.W, p.orders, cands, p.meta,
                                                              bad);
     } else {
-        cudaFuncSetAttribute(k_sweep_f32<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sw_smem);
+        allow_smem(k_sweep_f32<false>, sw_smem);
         StageTimer _t(STAGE_SWEEP, st);
         k_sweep_f32<false><<<blocks, 32 * spb, sw_smem, st>>>(p.skip, P, n, p.h, p.ev, p.range, p.W, p.orders, cands, p.meta,
                                                               bad);

@@ -56,3 +56,26 @@ def test_installed_workspace(H, n, dtype, algorithm):
     assert [r() for r in runs] == [0] * len(runs)
     H.set_workspace(buf, size - staging - 1)
     assert [r() for r in runs] == [6] * len(runs)   # LMS_ERR_WORKSPACE
+
+
+# ---------------------------------------------------------------- shared-memory limits
+def test_shared_memory_limits_are_only_raised(H):
+    """The limit of a kernel is shared by all host threads: a smaller call between another thread's limit and its
+    launch must not lower it (plans of different sizes, fits of different n)."""
+    sizes = {}
+
+    def calls():
+        for n in (4096, 600):
+            assert H.fit(n) == 0 and H.fit(n, 0, "sweep") == 0 and H.fit_bnb(n, stats=True) == 0
+            assert H.fit(n, dtype=F32) == 0
+            rc, plan, off = H.plan([n, n])
+            assert rc == 0 and H.fit_batched(plan, off) == 0
+            yield n
+            H.lib.lms_batch_plan_destroy(plan)
+
+    for n in calls():
+        limits = {k: H.lib.fake_limit(k.encode()) for k in set(H.kernels())}
+        for k, v in limits.items():
+            assert v >= sizes.get(k, 0), (n, k)
+        sizes.update(limits)
+    assert max(sizes.values()) > 48 * 1024
