@@ -223,7 +223,7 @@ cudaError_t allow_smem_of(const void *kernel, size_t bytes)
     int dev;
     if (current_device(dev)) return cudaErrorInvalidDevice;
     std::lock_guard<std::mutex> lock(mu);
-    size_t &limit = limits.try_emplace({dev, kernel}, (size_t)48 * 1024).first->second;
+    size_t &limit = limits[{dev, kernel}];   // 0: never set (the default of 48 KB includes the static memory)
     if (bytes <= limit) return cudaSuccess;
     const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
     if (e == cudaSuccess) limit = bytes;

@@ -15,7 +15,7 @@ namespace {
 
 struct Kernel {
     std::string name;
-    size_t limit = 48 * 1024;   // dynamic shared memory a launch may ask for
+    size_t limit = 44 * 1024;   // dynamic shared memory a launch may ask for (48 KB less what a kernel has of its own)
 };
 struct Launch {
     std::string name;
