@@ -51,6 +51,12 @@
 #include "kernels.cuh"
 #include "lms.h"
 
+// Counters of the host build that the tests make of this file (one thread a
+// group, T = G = 1): phases by mode and what each works on.
+#ifndef LMS_DIRECT_COUNT
+#define LMS_DIRECT_COUNT(what, n)
+#endif
+
 namespace lms {
 namespace {
 
@@ -66,6 +72,8 @@ constexpr int TABLE = 2048;                // slots of a CTA's slope table
 constexpr float LEAF_FRACTIONS = 32.0f;      // an interval with this few possible slopes is a leaf
 constexpr float FRACTIONS = 1000.0f;         // expected fractions of a leaf up to which they are tried one by one
 constexpr int CELLS_MAX = 8192;             // cells of the pair search
+constexpr float DENSE = 16384.0f;            // candidates up to which a leaf's pairs are searched in the cells ..
+constexpr float DENSE_PER_POINT = 64.0f;     // .. and so many more for each point (ordinary sets: at most 30 a point)
 constexpr int WIDE_ITEMS = 2;              // up to so many questions a CTA, the whole CTA works on each
 constexpr int DEPTH_MAX = 28;              // levels: an interval has fewer than 2^48 keys, NODE_F^24
 constexpr int F_SCORES = 4096;             // slopes of a float set that are scored, else the sweep takes over
@@ -85,7 +93,7 @@ enum Mode { M_TREE, M_PAIRS, M_EVENT, M_EXACT, M_DONE };
 // What the CTAs of a team share, in global memory.
 struct TeamState {
     long long ub;                // upper bound of the LMS value, units of 2^-32
-    int nlist[2], over[2];       // distinct slopes listed, overflow flag (by turns)
+    int nlist[2], over[2];       // distinct slopes listed (by turns); 1: too many, 2: too many candidates
     int bad;                     // a consistency check failed
     unsigned pair[2];            // smallest index pair of a slope (by turns)
 };
@@ -93,7 +101,7 @@ struct TeamState {
 // Answer to an interval test.
 struct Answer {
     long long t0, t1;
-    int keep, pad;
+    int keep, dense;   // dense: the pair search of a leaf was left out
 };
 
 // Best float candidate: lexicographic (w, theta1, theta2, pair).
@@ -111,6 +119,7 @@ struct TeamShape {
     int Q;       // root intervals
     float leaf;  // expected pairs of a leaf
     long long ptsn;   // points kept in global memory (0: in shared memory)
+    long long dupw;   // words of one bit a point
     long long sortw;  // bytes of global sort scratch per CTA
     int C;       // CTAs of a team
 };
@@ -129,6 +138,7 @@ struct TeamMem {
     unsigned *evd;
     Cand *xres;
     int *pts;
+    unsigned *dup;        // points that repeat an earlier one (marked when asked for)
     unsigned char *sort;
 };
 
@@ -137,7 +147,7 @@ __host__ __device__ inline long long team_bytes(const TeamShape &s)
     return d_up(sizeof(TeamState)) + d_up(sizeof(DNode) * (long long)stack_cap(s)) +
            d_up(sizeof(DNode) * (long long)estack_cap(s)) + d_up(2 * sizeof(Answer) * (long long)s.PM) +
            2 * d_up(8LL * s.HC) +
-           2 * d_up(4LL * s.HC) + d_up(sizeof(CandD) * (long long)s.PM) + d_up(4LL * s.ptsn) +
+           2 * d_up(4LL * s.HC) + d_up(sizeof(CandD) * (long long)s.PM) + d_up(4LL * s.ptsn) + d_up(4LL * s.dupw) +
            d_up(s.sortw) * s.C;
 }
 
@@ -155,6 +165,7 @@ __device__ inline TeamMem team_carve(unsigned char *p, const TeamShape &s)
     m.evd = reinterpret_cast<unsigned *>(take(4LL * s.HC));
     m.xres = reinterpret_cast<Cand *>(take(sizeof(CandD) * (long long)s.PM));   // or CandD
     m.pts = reinterpret_cast<int *>(take(4LL * s.ptsn));
+    m.dup = reinterpret_cast<unsigned *>(take(4LL * s.dupw));
     m.sort = p;
     return m;
 }
@@ -816,6 +827,22 @@ __device__ __forceinline__ int cta_scan_ex(int v, int *s_warp, int &total)
     }
 }
 
+// Whether the threads' values add up to more than limit (the same in every thread).
+template <int T>
+__device__ __forceinline__ bool candidates_above(float v, float limit, int *s_warp)
+{
+    if constexpr (T >= 32) {
+#pragma unroll
+        for (int d = 16; d >= 1; d >>= 1) v += __shfl_xor_sync(FULL, v, d);
+        if ((threadIdx.x & 31) == 0) s_warp[threadIdx.x >> 5] = __float_as_int(v);
+        __syncthreads();
+        v = 0.0f;
+        for (int w = 0; w < T / 32; ++w) v += __int_as_float(s_warp[w]);
+        __syncthreads();
+    }
+    return v > limit;
+}
+
 template <int T>
 __device__ __forceinline__ void cta_min_max_i(int &lo, int &hi, int *s_a, int *s_b)
 {
@@ -872,6 +899,47 @@ __device__ __forceinline__ void table_put(const SlopeTable &t, long long key, in
     }
 }
 
+template <int T>
+__device__ __forceinline__ SlopeTable table_clear(unsigned char *wk)
+{
+    SlopeTable t;
+    t.key = reinterpret_cast<unsigned long long *>(wk);
+    t.den = reinterpret_cast<unsigned *>(t.key + TABLE);
+    t.count = reinterpret_cast<int *>(t.den + TABLE);
+    for (int k = threadIdx.x; k < TABLE; k += T) t.key[k] = ~0ull;
+    if (threadIdx.x == 0) *t.count = 0;
+    return t;
+}
+
+// The table's slopes go to the end of the team's list; *over when they do not fit.
+template <int T>
+__device__ __forceinline__ void table_append(const SlopeTable &tab, const TeamMem &m, int *nlist, int *over, int HC,
+                                             int *s_warp)
+{
+    const int held = *tab.count;
+    __shared__ int s_at;
+    if (threadIdx.x == 0) {
+        s_at = held > TABLE * 3 / 4 ? HC : atomicAdd(nlist, held);
+        if (s_at + held > HC) atomicMax(over, 1);
+    }
+    __syncthreads();
+    int at = s_at;
+    if (at + held <= HC) {
+        const int per = TABLE / T;
+        int c = 0, total;
+        for (int r = 0; r < per; ++r) c += tab.key[threadIdx.x * per + r] != ~0ull;
+        at += cta_scan_ex<T>(c, s_warp, total);
+        for (int r = 0; r < per; ++r) {
+            const unsigned long long k = tab.key[threadIdx.x * per + r];
+            if (k != ~0ull) {
+                m.lkey[at] = (long long)k;
+                m.lden[at++] = tab.den[threadIdx.x * per + r];
+            }
+        }
+    }
+    __syncthreads();
+}
+
 // The dy of the slope with this key and dx: key <= dy 2^32 / dx < key + 1.
 __device__ __forceinline__ int dy_of(long long key, int dx)
 {
@@ -884,10 +952,25 @@ __device__ __forceinline__ unsigned gcd32(unsigned a, unsigned b)
     return a;
 }
 
-// Expected reduced fractions p / q in slope keys [A, B), q <= X.
-__device__ __forceinline__ float fractions(long long A, long long B, int xr)
+// Largest q of a fraction p / q with key in [A, B), q <= X and |p| <= Y.
+__device__ __forceinline__ int fraction_q(long long A, long long B, int xr, int yr)
 {
-    return 0.31f * (float)xr * (float)xr * (float)(B - A) * (1.0f / 4294967296.0f);
+    const long long nearest = A > 0 ? A : B < 0 ? -B : 0;
+    return nearest ? (int)min((long long)xr, (((long long)yr + 1) << 32) / nearest + 1) : xr;
+}
+
+// Expected reduced fractions p / q of such a leaf: about 0.31 q^2 times its width.
+__device__ __forceinline__ float fractions(long long A, long long B, int xr, int yr)
+{
+    const float q = (float)fraction_q(A, B, xr, yr);
+    return 0.31f * q * q * (float)(B - A) * (1.0f / 4294967296.0f);
+}
+
+// Slopes a leaf is expected to list: its pairs, or its fractions where those are tried.
+__device__ __forceinline__ float leaf_slopes(const DNode &lf, float gain, int xr, int yr)
+{
+    const float f = fractions(lf.a, lf.b, xr, yr), e = fmaxf(lf.est * gain, 1.0f);
+    return f < FRACTIONS ? fminf(f + 1.0f, 4.0f * e + LEAF_FRACTIONS) : e;
 }
 
 // Shared bytes of list_pairs for NC cells and n points.
@@ -905,19 +988,26 @@ __host__ __device__ constexpr size_t pairs_bytes(int NC, int n)
 // FRACTIONS of them the CTA tries every q.  p / q lies in the leaf when
 // g = -A q mod 2^32 is below (B - A) q: two 32-bit products a q, whatever the
 // number of points (n = 65536, 10 leaves: 4.6 ms by pairs).  Otherwise the
-// pairs are found by cells (see the head of the file).
+// pairs are found by cells (see the head of the file); so are they when the
+// leaves listed together hold more fractions than the list and this one far
+// more than the pairs expected (most fractions are then no pair's slope, and
+// each would be tested and scored).  Cells that hold many points hold
+// quadratically many candidates with few distinct slopes.  Above the limit
+// nothing is searched: points that repeat another one are left out (dup, once
+// they are marked: 2048 points, 70% of them at one place, cost 35 ms of
+// candidates), and for points on one line the leaf is tried by fractions, or
+// false is returned and it is cut until it can be.
 template <int T>
-__device__ __noinline__ void list_pairs(const int *pts, int n, long long A, long long B, const Box &bx, int NC,
-                                        unsigned char *wk, int *s_warp, const TeamMem &m,
+__device__ __noinline__ bool list_pairs(const int *pts, int n, const unsigned *dup, const DNode &lf, bool by_fractions,
+                                        const Box &bx, int NC, unsigned char *wk, int *s_warp, const TeamMem &m,
                                         int *nlist, int *over, int HC,
                                         int part, int parts)
 {
+    const long long A = lf.a, B = lf.b;
     const int xr = bx.xhi - bx.xlo, yr = bx.yhi - bx.ylo;
-    if (fractions(A, B, xr) < FRACTIONS) {
+    auto by_q = [&]() {
         const long long d = B - A;
-        // |p| <= y range
-        const long long nearest = A > 0 ? A : B < 0 ? -B : 0;
-        const int qmax = nearest ? (int)min((long long)xr, (((long long)yr + 1) << 32) / nearest + 1) : xr;
+        const int qmax = fraction_q(A, B, xr, yr);
         for (int q = 1 + part * T + (int)threadIdx.x; q <= qmax; q += T * parts) {
             const long long end = d * q;
             for (long long g = (unsigned)(0u - (unsigned)A * (unsigned)q); g < end; g += 1LL << 32) {
@@ -928,23 +1018,21 @@ __device__ __noinline__ void list_pairs(const int *pts, int n, long long A, long
                 if (at < HC) {
                     m.lkey[at] = slope_key(y, q);
                     m.lden[at] = (unsigned)q;
-                } else {
-                    *over = 1;
+                } else if (at == HC) {
+                    atomicMax(over, 1);
                 }
             }
         }
-        return;
+    };
+    const float fr = fractions(A, B, xr, yr);
+    if (fr < FRACTIONS && (by_fractions || fr <= 4.0f * fmaxf(lf.est, 1.0f) + LEAF_FRACTIONS)) {
+        by_q();
+        return true;
     }
-    SlopeTable tab;
-    tab.key = reinterpret_cast<unsigned long long *>(wk);
-    tab.den = reinterpret_cast<unsigned *>(tab.key + TABLE);
-    tab.count = reinterpret_cast<int *>(tab.den + TABLE);
+    auto out = [&](int k) { return dup && (__ldcg(&dup[k >> 5]) >> (k & 31) & 1); };
+    const SlopeTable tab = table_clear<T>(wk);
     unsigned *cnt = tab.den + TABLE + 4;
     unsigned short *ord = reinterpret_cast<unsigned short *>(cnt + NC);
-    for (int k = threadIdx.x; k < TABLE; k += T) {
-        tab.key[k] = ~0ull;
-    }
-    if (threadIdx.x == 0) *tab.count = 0;
     for (int q = threadIdx.x; q < NC; q += T) cnt[q] = 0u;
     __syncthreads();
     // beyond D_GUARD in units of 2^-26, the cells a little wider for the rounding
@@ -958,30 +1046,43 @@ __device__ __noinline__ void list_pairs(const int *pts, int n, long long A, long
         long long zlo, zhi;
         box_range(bx, za, ys, zlo, zhi);
         auto cell = [&](int p) { return (int)((unsigned long long)(z_at(p, za, ys) - zlo) >> sh) & (NC - 1); };
-        for (int k = threadIdx.x; k < n; k += T) atomicAdd(&cnt[cell(pts[k])], 1u);
+        for (int k = threadIdx.x; k < n; k += T)
+            if (!out(k)) atomicAdd(&cnt[cell(pts[k])], 1u);
         __syncthreads();
         const int per = NC / T;
         unsigned sum = 0;
-        for (int r = 0; r < per; ++r) sum += cnt[threadIdx.x * per + r];
-        int total;
-        unsigned run = (unsigned)cta_scan_ex<T>((int)sum, s_warp, total);
+        float cand = 0.0f;   // candidates: the rest of a cell, and the next cell
+        for (int r = 0; r < per; ++r) {
+            const unsigned c = cnt[threadIdx.x * per + r], c2 = cnt[(threadIdx.x * per + r + 1) & (NC - 1)];
+            sum += c;
+            cand += (float)c * (0.5f * (float)c + (float)c2);
+        }
+        if (candidates_above<T>(cand, DENSE + DENSE_PER_POINT * (float)n, s_warp)) {
+            // (every CTA that shares the leaf finds the same)
+            if (dup && fr < FRACTIONS) by_q();
+            __syncthreads();
+            return dup && fr < FRACTIONS;
+        }
+        int held;
+        unsigned run = (unsigned)cta_scan_ex<T>((int)sum, s_warp, held);
         for (int r = 0; r < per; ++r) {
             const unsigned c = cnt[threadIdx.x * per + r];
             cnt[threadIdx.x * per + r] = run;
             run += c;
         }
         __syncthreads();
-        for (int k = threadIdx.x; k < n; k += T) ord[atomicAdd(&cnt[cell(pts[k])], 1u)] = (unsigned short)k;
+        for (int k = threadIdx.x; k < n; k += T)
+            if (!out(k)) ord[atomicAdd(&cnt[cell(pts[k])], 1u)] = (unsigned short)k;
         __syncthreads();
         // cnt[q] is now the end of cell q, cnt[q - 1] its start.  A warp takes
         // 32 points at a time, lays their candidates (the rest of the cell,
         // then the next cell) end to end and tests 32 of them at once.
         constexpr int L = T >= 32 ? 32 : 1;
         const int lane = threadIdx.x % L;
-        for (int e0 = part * T + threadIdx.x - lane; e0 < n; e0 += T * parts) {
+        for (int e0 = part * T + threadIdx.x - lane; e0 < held; e0 += T * parts) {
             const int e = e0 + lane;
             int pa = 0, n1 = 0, nn = 0, beg2 = 0;
-            if (e < n) {
+            if (e < held) {
                 pa = pts[ord[e]];
                 const int q = cell(pa), q2 = (q + 1) & (NC - 1);
                 beg2 = q2 ? (int)cnt[q2 - 1] : 0;
@@ -997,6 +1098,7 @@ __device__ __noinline__ void list_pairs(const int *pts, int n, long long A, long
                 }
             }
             const int total = L == 32 ? __shfl_sync(FULL, pre, 31) : pre;
+            LMS_DIRECT_COUNT(M_DONE, total);
             for (int c0 = 0; c0 < total; c0 += L) {
                 const int c = c0 + lane;
                 int src = 0;   // the lane whose candidates hold c
@@ -1023,29 +1125,8 @@ __device__ __noinline__ void list_pairs(const int *pts, int n, long long A, long
         }
     }
     __syncthreads();
-    // append the table
-    const int held = *tab.count;
-    __shared__ int s_at;
-    if (threadIdx.x == 0) {
-        s_at = held > TABLE * 3 / 4 ? HC : atomicAdd(nlist, held);
-        if (s_at + held > HC) *over = 1;
-    }
-    __syncthreads();
-    int at = s_at;
-    if (at + held <= HC) {
-        const int per = TABLE / T;
-        int c = 0, total;
-        for (int r = 0; r < per; ++r) c += tab.key[threadIdx.x * per + r] != ~0ull;
-        at += cta_scan_ex<T>(c, s_warp, total);
-        for (int r = 0; r < per; ++r) {
-            const unsigned long long k = tab.key[threadIdx.x * per + r];
-            if (k != ~0ull) {
-                m.lkey[at] = (long long)k;
-                m.lden[at++] = tab.den[threadIdx.x * per + r];
-            }
-        }
-    }
-    __syncthreads();
+    table_append<T>(tab, m, nlist, over, HC, s_warp);
+    return true;
 }
 
 // ------------------------------------------------------------------ float points
@@ -1121,6 +1202,7 @@ __device__ __noinline__ void list_pairs_f32(const int2 *pts, int n, long long A,
         const int q = cell(pa), q2 = (q + 1) & (NC - 1);
         const int beg2 = q2 ? (int)cnt[q2 - 1] : 0;
         const int n1 = (int)cnt[q] - e - 1, nn = n1 + (int)cnt[q2] - beg2;
+        LMS_DIRECT_COUNT(M_DONE, nn);
         if (*reinterpret_cast<volatile int *>(over)) break;   // the leaf is cut instead
         for (int u = threadIdx.x % L; u < nn; u += L) {
             const int b = ord[u < n1 ? e + 1 + u : beg2 + u - n1];
@@ -1145,6 +1227,31 @@ __device__ __noinline__ void list_pairs_f32(const int2 *pts, int n, long long A,
     __syncthreads();
 }
 
+// The smallest width of the CTA's threads and the first window that has it.
+template <int T, class W>
+__device__ __forceinline__ void cta_first_min(W &bw, int &ba, long long *s_red)
+{
+    if constexpr (T >= 32) {
+#pragma unroll
+        for (int d = 16; d >= 1; d >>= 1) {
+            const W ow = __shfl_xor_sync(FULL, bw, d);
+            const int oa = __shfl_xor_sync(FULL, ba, d);
+            if (ow < bw || (ow == bw && oa < ba)) { bw = ow; ba = oa; }
+        }
+        if ((threadIdx.x & 31) == 0) {
+            s_red[2 * (threadIdx.x >> 5)] = (long long)bw;
+            s_red[2 * (threadIdx.x >> 5) + 1] = ba;
+        }
+        __syncthreads();
+        for (int w = 0; w < T / 32; ++w) {
+            const W ow = (W)s_red[2 * w];
+            const int oa = (int)s_red[2 * w + 1];
+            if (ow < bw || (ow == bw && oa < ba)) { bw = ow; ba = oa; }
+        }
+        __syncthreads();
+    }
+}
+
 // The narrowest window at the double slope s, as the float sweep computes it:
 // z = y - s x in double, w = z_hi - z_lo; ties take the lowest window.
 template <int T>
@@ -1167,25 +1274,7 @@ __device__ __noinline__ void score_f32(const FloatSet &f, int n, int h, double s
         const long long d = order_of(__dsub_rn(of_order(v[a + h - 1]), of_order(v[a])));
         if (d < bw) { bw = d; ba = a; }
     }
-    if constexpr (T >= 32) {
-#pragma unroll
-        for (int d = 16; d >= 1; d >>= 1) {
-            const long long ow = __shfl_xor_sync(FULL, bw, d);
-            const int oa = __shfl_xor_sync(FULL, ba, d);
-            if (ow < bw || (ow == bw && oa < ba)) { bw = ow; ba = oa; }
-        }
-        if ((threadIdx.x & 31) == 0) {
-            s_red[2 * (threadIdx.x >> 5)] = bw;
-            s_red[2 * (threadIdx.x >> 5) + 1] = ba;
-        }
-        __syncthreads();
-        for (int q = 0; q < T / 32; ++q) {
-            const long long ow = s_red[2 * q];
-            const int oa = (int)s_red[2 * q + 1];
-            if (ow < bw || (ow == bw && oa < ba)) { bw = ow; ba = oa; }
-        }
-        __syncthreads();
-    }
+    cta_first_min<T>(bw, ba, s_red);
     const double zb = of_order(v[ba]), zt = of_order(v[ba + h - 1]);
     w = zt - zb;
     t = 0.5 * (zb + zt);
@@ -1271,25 +1360,7 @@ __device__ void min_window(const W *s, int n, int h, W &bw, int &ba, long long *
         const W w = s[a + h - 1] - s[a];
         if (w < bw) { bw = w; ba = a; }
     }
-    if constexpr (T >= 32) {
-#pragma unroll
-        for (int d = 16; d >= 1; d >>= 1) {
-            const W ow = __shfl_xor_sync(FULL, bw, d);
-            const int oa = __shfl_xor_sync(FULL, ba, d);
-            if (ow < bw || (ow == bw && oa < ba)) { bw = ow; ba = oa; }
-        }
-        if ((threadIdx.x & 31) == 0) {
-            s_red[2 * (threadIdx.x >> 5)] = (long long)bw;
-            s_red[2 * (threadIdx.x >> 5) + 1] = ba;
-        }
-        __syncthreads();
-        for (int w = 0; w < T / 32; ++w) {
-            const W ow = (W)s_red[2 * w];
-            const int oa = (int)s_red[2 * w + 1];
-            if (ow < bw || (ow == bw && oa < ba)) { bw = ow; ba = oa; }
-        }
-        __syncthreads();
-    }
+    cta_first_min<T>(bw, ba, s_red);
 }
 
 template <int T>
@@ -1300,7 +1371,7 @@ __device__ __noinline__ Cand score(const int *pts, int n, int h, int dy, int dx,
     const long long lo = (long long)bx.ylo * dx - max(u, v), hi = (long long)bx.yhi * dx - min(u, v);
     int P = T;
     while (P < n) P <<= 1;
-    Cand c;
+    Cand c = cand_empty();
     c.dy = dy;
     c.dx = dx;
     // centred projections are (projection) - (yc dx - xc dy)
@@ -1452,6 +1523,44 @@ __device__ __noinline__ void line_pair(const int *pts, int n, int dy, int dx, un
                     break;
                 }
                 if (probe == slots) *bad = 1;   // the share did not fit: reported, never silent
+            }
+            __syncthreads();
+        }
+    }
+}
+
+// Sets the bit of every point that repeats one of a smaller index (the words
+// of dup are 0 before).  Table, rounds and shares as in line_pair.
+template <int T>
+__device__ __noinline__ void mark_duplicates(const int *pts, int n, unsigned *tab, int slots, int rounds, int part,
+                                             int parts, unsigned *dup, int *bad)
+{
+    for (int r = part; r < rounds; r += parts) {
+        __syncthreads();
+        for (int k = threadIdx.x; k < slots; k += T) tab[k] = ~0u;
+        __syncthreads();
+        for (int step = 0; step < 2; ++step) {
+            for (int k = threadIdx.x; k < n; k += T) {
+                const int p = pts[k];
+                const unsigned hs = mix32((unsigned)p);
+                if ((int)(hs & (unsigned)(rounds - 1)) != r) continue;
+                unsigned s = (hs >> 8) & (unsigned)(slots - 1);
+                int probe = 0;
+                for (; probe < slots; ++probe, s = (s + 1) & (unsigned)(slots - 1)) {
+                    unsigned cur = *reinterpret_cast<volatile unsigned *>(&tab[s]);
+                    if (cur == ~0u) {
+                        cur = atomicCAS(&tab[s], ~0u, (unsigned)k);
+                        if (cur == ~0u) break;
+                    }
+                    if (pts[cur] != p) continue;
+                    if (step == 0) {
+                        if (cur > (unsigned)k) atomicMin(&tab[s], (unsigned)k);
+                    } else if (cur != (unsigned)k) {
+                        atomicOr(&dup[k >> 5], 1u << (k & 31));
+                    }
+                    break;
+                }
+                if (probe == slots) *bad = 1;
             }
             __syncthreads();
         }
@@ -1799,9 +1908,15 @@ __global__ void __launch_bounds__(T) k_direct(const DirectArgs A)
             nd.est = nd.a < nd.b ? 0.5f * (float)n * (float)(n - 1) / (float)(Q + 1) : -1.0f;
             S.work[0][q] = nd;
         }
+        // hash tables of line_pair and mark_duplicates
+        int slots = 1024, rounds = 1;
+        while (slots * 8 <= wk_bytes && slots < 2 * n) slots <<= 1;
+        while (rounds < (int)C || (long long)rounds * slots < 2LL * n) rounds <<= 1;
         // the plan: the same values in every thread of the team
         int mode = M_TREE, P = Q + 1, cur = 0, par = 0, lpar = 0, ppar = 0;
-        int top = 0, etop = 0, nleaf = 0, lf0 = 0, lfn = 0, nx = 0, err = 0, regrown = 0, scored = 0;
+        int top = 0, etop = 0, nleaf = 0, lf0 = 0, lfn = 0, nx = 0, err = 0, regrown = 0, scored = 0, lcap = LC;
+        float gain = 1.0f;
+        [[maybe_unused]] bool marked = false;   // duplicates are marked
         bool flush = false;
         long long ux = D_MAX, uxl = D_MAX, bkey = D_MAX;
         Cand best = cand_empty();
@@ -1809,6 +1924,7 @@ __global__ void __launch_bounds__(T) k_direct(const DirectArgs A)
         team_sync();
         for (int phase = 0; mode != M_DONE; ++phase) {
             DNode *work = S.work[cur], *next = S.work[cur ^ 1];
+            LMS_DIRECT_COUNT(mode, mode == M_EXACT ? nx : mode == M_PAIRS ? lfn : P);
             if (mode == M_TREE || mode == M_EVENT) {
                 const bool ev = mode == M_EVENT;
                 // ------------------------------------------------ interval tests
@@ -1884,7 +2000,8 @@ __global__ void __launch_bounds__(T) k_direct(const DirectArgs A)
                     if (nd.b > -(D_GUARD - 1) && nd.a <= -D_GUARD) return false;
                     if (nd.b - nd.a == 1) return true;
                     if (nd.force > 0) return false;
-                    return nd.est <= sh.leaf || (!F && fractions(nd.a, nd.b, xr) <= LEAF_FRACTIONS);
+                    const float f = F ? 0.0f : fractions(nd.a, nd.b, xr, yr);
+                    return nd.est * gain <= sh.leaf || (!F && f <= LEAF_FRACTIONS);
                 };
                 const int pers = (ns + T - 1) / T;
                 const int i0 = min(ns, (int)threadIdx.x * pers), i1 = min(ns, i0 + pers);
@@ -1956,18 +2073,51 @@ __global__ void __launch_bounds__(T) k_direct(const DirectArgs A)
                 int NC = T;
                 while (NC < n && NC < CELLS_MAX) NC <<= 1;
                 const int parts = max(1, (int)C / lfn);
+                [[maybe_unused]] bool by_fractions = true;
+                if constexpr (!F) {
+                    float held = 0.0f;
+                    for (int l = lf0; l < lf0 + lfn; ++l) {
+                        const float f = fractions(S.leaf[l].a, S.leaf[l].b, xr, yr);
+                        if (f < FRACTIONS) held += f;
+                    }
+                    by_fractions = held <= 0.75f * (float)sh.HC;
+                }
                 for (int l = rank; l < lfn * parts; l += C) {
                     const DNode &lf = S.leaf[lf0 + l / parts];
                     if constexpr (F)
                         list_pairs_f32<T>(pts, n, lf.a, lf.b, bx, fs, NC, wk, S.warp_a, m, &st->nlist[lpar],
                                           &st->over[lpar], sh.HC, l % parts, parts);
-                    else
-                        list_pairs<T>(pts, n, lf.a, lf.b, bx, NC, wk, S.warp_a, m, &st->nlist[lpar], &st->over[lpar],
-                                      sh.HC, l % parts, parts);
+                    else {
+                        const bool listed = list_pairs<T>(pts, n, marked ? m.dup : nullptr, lf, by_fractions, bx, NC, wk,
+                                                          S.warp_a, m, &st->nlist[lpar], &st->over[lpar], sh.HC,
+                                                          l % parts, parts);
+                        if (threadIdx.x == 0 && l % parts == 0) {
+                            m.ans[l / parts].dense = !listed;   // (no test runs here; LC <= 2 PM answers)
+                            if (!listed && !marked) atomicMax(&st->over[lpar], 2);
+                        }
+                    }
                 }
                 team_sync();
-                const bool over = __ldcg(&st->over[lpar]) != 0;
+                const int over = __ldcg(&st->over[lpar]);
                 const int nn = __ldcg(&st->nlist[lpar]);
+                // slopes to expect for each pair expected: few where many pairs share a slope
+                {
+                    float held = 0.0f;
+                    for (int l = lf0; l < lf0 + lfn; ++l)
+                        held += F ? S.leaf[l].est * gain : leaf_slopes(S.leaf[l], gain, xr, yr);
+                    if (over) gain = fminf(1.0f, 4.0f * gain);
+                    else if (8.0f * (float)nn < held) gain = fmaxf(1.0f / 4096, 0.25f * gain);
+                }
+                if constexpr (!F) {
+                    if (over == 2) {
+                        // the first leaf with too many candidates: duplicates are marked, the leaves listed again
+                        for (int k = rank * T + threadIdx.x; k < (n + 31) / 32; k += T * C) m.dup[k] = 0u;
+                        team_sync();
+                        mark_duplicates<T>(pts, n, reinterpret_cast<unsigned *>(wk), slots, rounds, (int)rank, (int)C,
+                                           m.dup, &st->bad);
+                        marked = true;
+                    }
+                }
                 if (rank == 0 && !over) {
                     long long *s = reinterpret_cast<long long *>(wk);
                     if (nn <= 512) {
@@ -2032,11 +2182,31 @@ __global__ void __launch_bounds__(T) k_direct(const DirectArgs A)
                         S.work[cur][q] = nd;
                     }
                     P = runs;
+                    lcap = min(2 * lcap, LC);
+                    if constexpr (!F) {
+                        // leaves with too many candidates are cut before they are listed again
+                        int any = 0;
+                        for (int l = threadIdx.x; l < lfn; l += T) any |= __ldcg(&m.ans[l].dense);
+                        if (__syncthreads_or(any)) {
+                            int dense = 0;
+                            for (int l = 0; l < lfn; ++l) dense += __ldcg(&m.ans[l].dense);
+                            if (top + dense > stack_cap(sh)) err = 1;
+                            for (int l = lfn - 1, at = top; l >= 0 && !err && rank == 0 && threadIdx.x == 0; --l)
+                                if (__ldcg(&m.ans[l].dense)) {
+                                    DNode nd = S.leaf[lf0 + l];
+                                    nd.force = 2;
+                                    m.stack[at++] = nd;
+                                }
+                            top += dense;
+                        }
+                    }
                     lf0 += lfn;
                     if (lf0 == nleaf) {
                         lf0 = nleaf = 0;
                         flush = false;
                     }
+                } else if (over == 2) {
+                    P = 0;
                 } else if (lfn > 1 && regrown < (F ? 8 : 2) && lfn <= PM && lfn == nleaf) {
                     // their expected pairs were too low: cut them once more
                     for (int j = threadIdx.x; j < lfn; j += T) {
@@ -2049,7 +2219,7 @@ __global__ void __launch_bounds__(T) k_direct(const DirectArgs A)
                     nleaf = 0;
                     flush = false;
                 } else if (lfn > 1) {
-                    lfn = max(1, lfn / 4);
+                    lfn = lcap = max(1, lfn / 4);
                     P = 0;
                 } else {
                     // one leaf with too many slopes: more intervals of it, the other leaves wait on the stack
@@ -2122,10 +2292,6 @@ __global__ void __launch_bounds__(T) k_direct(const DirectArgs A)
                 }
                 team_sync();
                 // the best of them that is a pair's slope (fractions need not be)
-                int slots = 1024;
-                while (slots * 8 <= wk_bytes && slots < 2 * n) slots <<= 1;
-                int rounds = 1;
-                while (rounds < (int)C || (long long)rounds * slots < 2LL * n) rounds <<= 1;
                 for (int tries = 0; tries < nx; ++tries) {
                     Cand c = cand_empty();
                     int at = -1;
@@ -2185,7 +2351,17 @@ __global__ void __launch_bounds__(T) k_direct(const DirectArgs A)
                     top += P;
                     P = 0;
                 }
-                lfn = nleaf - lf0;
+                // as many of the leaves as the list is expected to hold
+                lfn = min(nleaf - lf0, lcap);
+                {
+                    float held = 0.0f;
+                    int l = 0;
+                    for (; l < lfn; ++l) {
+                        held += F ? fmaxf(S.leaf[lf0 + l].est * gain, 1.0f) : leaf_slopes(S.leaf[lf0 + l], gain, xr, yr);
+                        if (l > 0 && held > 0.75f * (float)sh.HC) break;
+                    }
+                    lfn = max(1, l);
+                }
                 flush = true;
             } else if (was_tree && P > 0) {
                 mode = M_TREE;
@@ -2276,6 +2452,7 @@ struct Shape {
         t.Q = std::min(PM, 128) - 1;
         t.leaf = leaf;
         t.ptsn = SP_ ? 0 : (long long)nmax * (PT / 4);
+        t.dupw = F_ ? 0 : (nmax + 31) / 32;
         t.sortw = 16LL * std::max<long long>(P, HC);
         t.C = C;
         return t;

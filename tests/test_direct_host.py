@@ -1,0 +1,47 @@
+"""The one-kernel branch-and-bound run on the host (direct_host.py): its
+records equal the oracle's, and sets whose pairs share slopes or whose slopes
+share widths take no more than a bounded amount of work."""
+import numpy as np
+import pytest
+
+import direct_host
+from direct_sets import points
+
+EXACT = ("status", "w_num", "w_den", "s_num", "s_den", "t_num", "t_den", "i", "j")
+
+
+@pytest.fixture(scope="module")
+def D(tmp_path_factory):
+    return direct_host.load(tmp_path_factory.mktemp("direct"))
+
+
+@pytest.mark.parametrize("kind", ["line", "sloped", "pure", "random", "full", "columns", "rows", "vertical", "lattice",
+                                  "digital", "collinear", "two_lines", "equal_x", "duplicates"])
+def test_int16_equals_oracle(D, orc, kind):
+    for n in (2, 3, 7, 33, 64, 65, 129, 300):
+        x, y = points(kind, n, 3 * n)
+        x, y = x.astype(np.int16), y.astype(np.int16)
+        for h in sorted({1, 2, n // 8 + 1, n // 2 + 1, int(0.75 * n) + 1, n} & set(range(1, n + 1))):
+            want = orc.lms_i16(x, y, h, "brute" if n <= 160 else "sweep")
+            for batch in (False, True):
+                r, _ = D.i16(x, y, h, batch)
+                assert tuple(int(r[k]) for k in EXACT) == tuple(want.exact()), (kind, n, h, batch, r, want)
+
+
+# The counters of ordinary sets at these sizes: at most 16 phases, 32 candidates a point and leaf, 10 slopes scored.
+@pytest.mark.parametrize("kind,n,h", [("duplicates", 2048, 0), ("duplicates", 513, 0), ("two_lines", 4096, 4096),
+                                      ("pure", 2048, 267), ("rows", 2048, 0), ("collinear", 4096, 0)])
+def test_shared_slopes_take_bounded_work(D, kind, n, h):
+    """Duplicates and points on few lines: the candidates of the pair search and the phases stay bounded (the pairs in
+    one cell are quadratically many, with few distinct slopes)."""
+    _, c = D.i16(*points(kind, n, n), h)
+    assert c["phases"] <= 64, c
+    assert c["candidates_sum"] <= 4096 * n, c
+    assert c["exact_sum"] <= 512, c
+
+
+def test_shared_widths_are_not_scored_as_fractions(D):
+    """Points in few columns: many slopes share the width; only slopes of pairs are scored (they were 253,056
+    fractions, most of them no pair's slope)."""
+    _, c = D.i16(*points("vertical", 8192, 8192), 6144)
+    assert c["exact_sum"] <= 16384 and c["phases"] <= 256, c
