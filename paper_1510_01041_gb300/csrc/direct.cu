@@ -74,10 +74,13 @@ constexpr float FRACTIONS = 1000.0f;         // expected fractions of a leaf up 
 constexpr int CELLS_MAX = 8192;             // cells of the pair search
 constexpr float DENSE = 16384.0f;            // candidates up to which a leaf's pairs are searched in the cells ..
 constexpr float DENSE_PER_POINT = 64.0f;     // .. and so many more for each point (ordinary sets: at most 30 a point)
+constexpr float F_DENSE = 8388608.0f;        // .. of a float set, which is left to the sweep beyond (no fractions there)
 constexpr int WIDE_ITEMS = 2;              // up to so many questions a CTA, the whole CTA works on each
 constexpr int DEPTH_MAX = 28;              // levels: an interval has fewer than 2^48 keys, NODE_F^24
-constexpr int F_SCORES = 4096;             // slopes of a float set that are scored, else the sweep takes over
-constexpr int F_PHASES = 400;
+// A float set is left to the sweep beyond these (ordinary sets: at most 13 phases, 1 cut, 130 slopes scored).
+constexpr int F_SCORES = 256;              // slopes scored
+constexpr int F_PHASES = 48;
+constexpr int F_CUTS = 3;                  // lists that did not hold their leaves' slopes
 constexpr int PHASES_MAX = 1 << 20;        // phases of one fit before it is reported as failed
 constexpr int EV_DEPTH = 6;                // levels of a run of at most EV_F^EV_DEPTH slopes
 
@@ -1158,16 +1161,20 @@ __device__ __forceinline__ double z_f32(const FloatSet &f, int k, double s)
     return __dsub_rn((double)f.y[k], __dmul_rn(s, (double)f.x[k]));
 }
 
-// The pairs whose slope lies in the leaf [A, B) of scaled slope keys, listed
-// by one CTA's share: slope bits and index pair.  Cells of z(A) as in
+// The distinct slopes of the pairs in the leaf [A, B) of scaled slope keys
+// (their order_of words), listed by one CTA's share; with `want` instead the
+// smallest index pair of that slope, lowered into *pair.  Cells of z(A) as in
 // list_pairs; both points of a pair may lie half a step off the grid in x and
-// y, which widens the cells by (1 + |s|) steps.
+// y, which widens the cells by (1 + |s|) steps.  *over = 2 (nothing listed)
+// when the cells hold too many candidates.
 template <int T>
 __device__ __noinline__ void list_pairs_f32(const int2 *pts, int n, long long A, long long B, const Box &bx,
                                             const FloatSet &f, int NC, unsigned char *wk, int *s_warp,
-                                            const TeamMem &m, int *nlist, int *over, int HC, int part, int parts)
+                                            const TeamMem &m, int *nlist, int *over, int HC, int part, int parts,
+                                            const long long *want = nullptr, unsigned *pair = nullptr)
 {
-    unsigned *cnt = reinterpret_cast<unsigned *>(wk);
+    const SlopeTable tab = table_clear<T>(wk);
+    unsigned *cnt = tab.den + TABLE + 4;
     unsigned short *ord = reinterpret_cast<unsigned short *>(cnt + NC);
     for (int q = threadIdx.x; q < NC; q += T) cnt[q] = 0u;
     __syncthreads();
@@ -1183,7 +1190,17 @@ __device__ __noinline__ void list_pairs_f32(const int2 *pts, int n, long long A,
     __syncthreads();
     const int per = NC / T;
     unsigned sum = 0;
-    for (int r = 0; r < per; ++r) sum += cnt[threadIdx.x * per + r];
+    float cand = 0.0f;
+    for (int r = 0; r < per; ++r) {
+        const unsigned c = cnt[threadIdx.x * per + r], c2 = cnt[(threadIdx.x * per + r + 1) & (NC - 1)];
+        sum += c;
+        cand += (float)c * (0.5f * (float)c + (float)c2);
+    }
+    if (candidates_above<T>(cand, F_DENSE, s_warp) && !want) {
+        if (threadIdx.x == 0) atomicMax(over, 2);
+        __syncthreads();
+        return;
+    }
     int total;
     unsigned run = (unsigned)cta_scan_ex<T>((int)sum, s_warp, total);
     for (int r = 0; r < per; ++r) {
@@ -1203,7 +1220,7 @@ __device__ __noinline__ void list_pairs_f32(const int2 *pts, int n, long long A,
         const int beg2 = q2 ? (int)cnt[q2 - 1] : 0;
         const int n1 = (int)cnt[q] - e - 1, nn = n1 + (int)cnt[q2] - beg2;
         LMS_DIRECT_COUNT(M_DONE, nn);
-        if (*reinterpret_cast<volatile int *>(over)) break;   // the leaf is cut instead
+        if (*reinterpret_cast<volatile int *>(tab.count) > TABLE * 3 / 4) break;   // the leaf is cut instead
         for (int u = threadIdx.x % L; u < nn; u += L) {
             const int b = ord[u < n1 ? e + 1 + u : beg2 + u - n1];
             const int2 pb = pts[b];
@@ -1215,16 +1232,16 @@ __device__ __noinline__ void list_pairs_f32(const int2 *pts, int n, long long A,
             if (!slope_f32(f, a, b, s)) continue;
             const double k = s * f.ratio * (double)(1LL << F_YS);
             if (!(k >= (double)A && k < (double)B)) continue;
-            const int at = atomicAdd(nlist, 1);
-            if (at < HC) {
-                m.lkey[at] = order_of(s);
-                m.lden[at] = (unsigned)min(a, b) << 16 | (unsigned)max(a, b);
+            if (want) {
+                const unsigned ij = (unsigned)min(a, b) << 16 | (unsigned)max(a, b);
+                if (order_of(s) == *want && *reinterpret_cast<volatile unsigned *>(pair) > ij) atomicMin(pair, ij);
             } else {
-                *over = 1;
+                table_put(tab, order_of(s), 0);
             }
         }
     }
     __syncthreads();
+    if (!want) table_append<T>(tab, m, nlist, over, HC, s_warp);
 }
 
 // The smallest width of the CTA's threads and the first window that has it.
@@ -1898,6 +1915,12 @@ __global__ void __launch_bounds__(T) k_direct(const DirectArgs A)
                 for (int i = gi; i < ns; i += NG) refine(g, std::integral_constant<int, NB>(), hist, i);
             }
         }
+        if constexpr (F) {
+            // steep slopes that stay in reach even at half the bound make the attempt useless
+            team_sync();
+            const long long U = __ldcg(&st->ub) / 2;
+            if (!steep_above_at(F_KMAX, bx.dh, yr, U < D_MAX / 4 ? U + grid_err(F_KMAX) : D_MAX)) return;
+        }
         for (int q = threadIdx.x; q <= Q; q += T) {
             DNode nd;
             nd.a = q == 0 ? -kmax : cut(q - 1);
@@ -1916,6 +1939,7 @@ __global__ void __launch_bounds__(T) k_direct(const DirectArgs A)
         int mode = M_TREE, P = Q + 1, cur = 0, par = 0, lpar = 0, ppar = 0;
         int top = 0, etop = 0, nleaf = 0, lf0 = 0, lfn = 0, nx = 0, err = 0, regrown = 0, scored = 0, lcap = LC;
         float gain = 1.0f;
+        [[maybe_unused]] int cuts_more = 0;
         [[maybe_unused]] bool marked = false;   // duplicates are marked
         bool flush = false;
         long long ux = D_MAX, uxl = D_MAX, bkey = D_MAX;
@@ -2105,6 +2129,8 @@ __global__ void __launch_bounds__(T) k_direct(const DirectArgs A)
                     float held = 0.0f;
                     for (int l = lf0; l < lf0 + lfn; ++l)
                         held += F ? S.leaf[l].est * gain : leaf_slopes(S.leaf[l], gain, xr, yr);
+                    if (F && (over == 2 || (over && (++cuts_more > F_CUTS || (lfn == 1 && S.leaf[lf0].b - S.leaf[lf0].a == 1)))))
+                        err = 1;   // more slopes or candidates than the sweep is worth
                     if (over) gain = fminf(1.0f, 4.0f * gain);
                     else if (8.0f * (float)nn < held) gain = fmaxf(1.0f / 4096, 0.25f * gain);
                 }
@@ -2256,7 +2282,7 @@ __global__ void __launch_bounds__(T) k_direct(const DirectArgs A)
                     for (int k = rank; k < nx && !err; k += C) {
                         CandD c;
                         c.s = of_order(__ldcg(&m.ev[S.xl[k]]));
-                        c.pair = __ldcg(&m.evd[S.xl[k]]);
+                        c.pair = 0;   // found for the best slope alone
                         c.valid = 1;
                         score_f32<T>(fs, n, h, c.s, wk, wk_bytes, gsort, S.red, c.w, c.t);
                         if (threadIdx.x == 0) reinterpret_cast<CandD *>(m.xres)[k] = c;
@@ -2268,7 +2294,7 @@ __global__ void __launch_bounds__(T) k_direct(const DirectArgs A)
                         c.w = __ldcg(&q->w);
                         c.s = __ldcg(&q->s);
                         c.t = __ldcg(&q->t);
-                        c.pair = __ldcg(&q->pair);
+                        c.pair = 0;
                         c.valid = 1;
                         if (candd_better(c, bestd)) bestd = c;
                     }
@@ -2376,25 +2402,16 @@ __global__ void __launch_bounds__(T) k_direct(const DirectArgs A)
             }
         }
         if constexpr (F) {
-            // the smallest index pair with the best slope: its pairs listed once more
-            if (rank == 0 && threadIdx.x == 0) st->nlist[lpar] = st->over[lpar] = 0;
-            team_sync();
+            // the smallest index pair with the best slope
             if (bestd.valid && !err) {
                 int NC = T;
                 while (NC < n && NC < CELLS_MAX) NC <<= 1;
-                const long long K = grid_key(bestd.s);
+                const long long K = grid_key(bestd.s), want = order_of(bestd.s);
                 list_pairs_f32<T>(pts, n, K - 1, K + 2, bx, fs, NC, wk, S.warp_a, m, &st->nlist[lpar], &st->over[lpar],
-                                  sh.HC, (int)rank, (int)C);
-            }
-            team_sync();
-            if (rank == 0 && bestd.valid && !err) {
-                const int nn = min(__ldcg(&st->nlist[lpar]), sh.HC);
-                int first = 0x7fffffff, last = 0;
-                for (int k = threadIdx.x; k < nn; k += T)
-                    if (__ldcg(&m.lkey[k]) == order_of(bestd.s)) first = min(first, (int)__ldcg(&m.lden[k]));
-                cta_min_max_i<T>(first, last, S.warp_a, S.warp_b);
-                if (__ldcg(&st->over[lpar])) err = 1;
-                else bestd.pair = (unsigned)first;
+                                  sh.HC, (int)rank, (int)C, &want, &st->pair[0]);
+                team_sync();
+                bestd.pair = __ldcg(&st->pair[0]);
+                if (bestd.pair == 0xffffffffu) err = 1;
             }
             // slopes beyond the tree's range must be out of reach
             const long long U = min(__ldcg(&st->ub), ux);

@@ -45,3 +45,55 @@ def test_shared_widths_are_not_scored_as_fractions(D):
     fractions, most of them no pair's slope)."""
     _, c = D.i16(*points("vertical", 8192, 8192), 6144)
     assert c["exact_sum"] <= 16384 and c["phases"] <= 256, c
+
+
+# ---------------------------------------------------------------- float sets
+def best_line(x, y, h):
+    """(w, theta1, theta2, pair) of the narrowest window over all pair slopes, computed as the float sweep does:
+    slopes and projections in double, the first in the order (w, theta1, theta2, pair)."""
+    x, y = x.astype(np.float64), y.astype(np.float64)
+    n = x.size
+    h = h or n // 2 + 1
+    i, j = np.triu_indices(n, 1)
+    dx, dy = x[j] - x[i], y[j] - y[i]
+    ok = dx != 0
+    i, j, dx, dy = i[ok], j[ok], dx[ok], dy[ok]
+    s = np.where(dx < 0, -dy, dy) / np.abs(dx)
+    best = None
+    for k in range(0, s.size, 4096):
+        z = np.sort(y[None] - s[k:k + 4096, None] * x[None], axis=1)
+        w = z[:, h - 1:] - z[:, :n - h + 1]
+        a = w.argmin(axis=1)
+        r = np.arange(a.size)
+        lo, hi = z[r, a], z[r, a + h - 1]
+        for q in np.flatnonzero(w[r, a] == w[r, a].min()):
+            c = (hi[q] - lo[q], s[k + q], 0.5 * (lo[q] + hi[q]), (int(i[k + q]), int(j[k + q])))
+            best = c if best is None or c < best else best
+    return best
+
+
+def check_float(D, x, y, h):
+    done, r, c = D.f32(x, y, h)
+    if done:
+        w, s, t, pair = best_line(np.float32(x), np.float32(y), h)
+        assert (r["theta1"], (r["i"], r["j"])) == (s, pair) and r["theta2"] == t, (x.size, h, r, (w, s, t, pair))
+        assert r["med_sq"] == (0.5 * w) * (0.5 * w)
+    return done, c
+
+
+@pytest.mark.parametrize("kind", ["line", "pure", "full", "columns", "rows", "lattice", "digital", "collinear",
+                                  "two_lines", "vertical", "duplicates"])
+def test_float_equals_sweep_arithmetic(D, kind):
+    """Integer coordinates as floats: ties of slopes and widths; an attempt that is given up is the sweep's."""
+    for n in (16, 33, 64, 160):
+        x, y = points(kind, n, 5 * n)
+        for h in (0, int(0.75 * n), int(0.4 * n)):
+            check_float(D, x, y, h)
+
+
+@pytest.mark.parametrize("kind", ["line", "digital", "collinear", "rows", "two_lines"])
+@pytest.mark.parametrize("n", [512, 2048])
+def test_float_shared_slopes_finish(D, kind, n):
+    """Pairs that share a slope are listed once (a leaf of one slope key overflowed its list: 403 phases, given up)."""
+    done, _, c = D.f32(*points(kind, n, n))
+    assert done and c["phases"] <= 24, c
