@@ -82,6 +82,8 @@ constexpr int F_SCORES = 256;              // slopes scored
 constexpr int F_PHASES = 48;
 constexpr int F_CUTS = 3;                  // lists that did not hold their leaves' slopes
 constexpr int PHASES_MAX = 1 << 20;        // phases of one fit before it is reported as failed
+constexpr int RUN_MIN = 12;                // slopes a CTA scores from which it keeps the points sorted between them
+constexpr int EXCHANGES = 16;              // passes that repair their order, else they are sorted again
 constexpr int EV_DEPTH = 6;                // levels of a run of at most EV_F^EV_DEPTH slopes
 
 struct DNode {
@@ -1500,6 +1502,85 @@ __device__ __noinline__ bool score_bins(const Group<T> &g, const int *pts, int n
     return false;
 }
 
+// The order of the points along slope dy/dx: words (projection, index),
+// ascending, in shared memory where they fit, else in gs (32 bytes a point).
+template <int T>
+__device__ __noinline__ unsigned long long *sort_points(const int *pts, int n, int dy, int dx, const Box &bx,
+                                                        unsigned char *wk, int wk_bytes, unsigned char *gs)
+{
+    const long long u = (long long)bx.xlo * dy, v = (long long)bx.xhi * dy;
+    const long long lo = (long long)bx.ylo * dx - max(u, v);
+    int P = T;
+    while (P < n) P <<= 1;
+    auto key = [&](int k) {   // projections span less than 2^34
+        return k < n ? (unsigned long long)(proj(pts[k], dy, dx) - lo) << 16 | (unsigned)k : 0xffffffffffffffffull;
+    };
+    unsigned long long *s = reinterpret_cast<unsigned long long *>(wk);
+    if (2 * P * 8 <= wk_bytes && P <= 16 * T) {
+        cta_fill_merge_sort_any(s, s + P, P, key);
+        return s;
+    }
+    unsigned long long *g = reinterpret_cast<unsigned long long *>(gs);
+    return cta_sort_chunked<4 * T>(s, g, g + P, P, key);
+}
+
+// The narrowest windows at count slopes in ascending order (their indices in
+// idx), one CTA: the points stay sorted from one slope to the next.  Where
+// the slopes that survive are dense (widths that many slopes share: points in
+// a few columns, near-vertical lines), few points change places between two
+// of them, so the order is repaired by odd-even exchanges (two or three
+// passes over the points) and every width is read off it, instead of two or
+// three histogram passes with their scans for each slope.
+template <int T>
+__device__ __noinline__ void score_run(const int *pts, int n, int h, const long long *ev, const unsigned *evd,
+                                       const int *idx, int count, const Box &bx, unsigned char *wk, int wk_bytes,
+                                       unsigned char *gs, long long *s_red, Cand *out)
+{
+    unsigned long long *s = nullptr;
+    for (int k = 0; k < count; ++k) {
+        const int dx = (int)__ldcg(&evd[idx[k]]), dy = dy_of(__ldcg(&ev[idx[k]]), dx);
+        bool sorted = false;
+        for (int it = 0; s != nullptr && it < EXCHANGES; ++it) {
+            int moved = 0;
+            for (int odd = 0; odd < 2; ++odd) {
+                for (int p = 2 * (int)threadIdx.x + odd; p + 1 < n; p += 2 * T) {
+                    const unsigned long long a = s[p], b = s[p + 1];
+                    const int pa = pts[a & 0xffffu], pb = pts[b & 0xffffu];
+                    if (proj(pb, dy, dx) < proj(pa, dy, dx)) {
+                        s[p] = b;
+                        s[p + 1] = a;
+                        moved = 1;
+                    }
+                }
+                __syncthreads();
+            }
+            if (!__syncthreads_or(moved)) {
+                sorted = true;
+                break;
+            }
+        }
+        if (!sorted) s = sort_points<T>(pts, n, dy, dx, bx, wk, wk_bytes, gs);
+        __syncthreads();
+        long long bw = D_MAX;
+        int ba = 0x7fffffff;
+        for (int a = threadIdx.x; a + h - 1 < n; a += T) {
+            const long long w = proj(pts[s[a + h - 1] & 0xffffu], dy, dx) - proj(pts[s[a] & 0xffffu], dy, dx);
+            if (w < bw) { bw = w; ba = a; }
+        }
+        cta_first_min<T>(bw, ba, s_red);
+        if (threadIdx.x == 0) {
+            Cand c = cand_empty();
+            c.dy = dy;
+            c.dx = dx;
+            c.w = bw;
+            // centred projections are (projection) - (yc dx - xc dy)
+            c.t = 2 * proj(pts[s[ba] & 0xffffu], dy, dx) + bw + 2 * ((long long)bx.yc * dx - (long long)bx.xc * dy);
+            out[k] = c;
+        }
+        __syncthreads();
+    }
+}
+
 // The smallest index pair (i < j) with slope dy/dx, lowered into *out (a
 // pair is i << 16 | j).  Points on one line of that slope share y dx - x dy; a
 // table in shared memory keeps the smallest index of every line, then each
@@ -2306,6 +2387,11 @@ __global__ void __launch_bounds__(T) k_direct(const DirectArgs A)
                         bkey = order_of(bestd.s);
                     }
                 } else {
+                const int r0 = (int)((long long)nx * rank / C), r1 = (int)((long long)nx * (rank + 1) / C);
+                if (nx >= RUN_MIN * (int)C)
+                    score_run<T>(pts, n, h, m.ev, m.evd, S.xl + r0, r1 - r0, bx, wk, wk_bytes, gsort, S.red,
+                                 m.xres + r0);
+                else
                 for (int k = rank; k < nx; k += C) {
                     const int dx = (int)__ldcg(&m.evd[S.xl[k]]), dy = dy_of(__ldcg(&m.ev[S.xl[k]]), dx);
                     Cand c;
