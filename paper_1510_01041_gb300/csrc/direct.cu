@@ -1139,6 +1139,7 @@ struct FloatSet {
     const float *x, *y;
     double xc, yc, sx, sy;   // grid = rint((v - c) * s), s a power of two
     double ratio;            // scaled slope = slope * ratio
+    double rx, ry;           // rounding of a width in double: rx |K| + ry units of 2^-F_YS steps
 };
 
 __device__ __forceinline__ long long order_of(double v)
@@ -1356,6 +1357,12 @@ __device__ bool float_box(const float *x, const float *y, int n, FloatSet &f, Bo
     f.sx = ldexp(1.0, F_BITS + 1 - ex);
     f.sy = ldexp(1.0, F_BITS + 1 - ey);
     f.ratio = ldexp(1.0, ex - ey);
+    // A projection y - s x computed in double is off by at most 2^-53 (|s x| +
+    // |y - s x|), a width of two of them by 2^-52 (2 |s x| + |y|) and its own
+    // rounding, far below one unit; 2^-51 covers both.  Not small beside the
+    // grid: points 2^22 of their spread away from the origin move by two steps.
+    f.rx = ldexp(fmax(fabs((double)xl), fabs((double)xh)) * f.sx, -50);
+    f.ry = ldexp(fmax(fabs((double)yl), fabs((double)yh)) * f.sy, F_YS - 51);
     if (threadIdx.x == 0) {
         bx.xc = bx.yc = bx.dh = 0;
         bx.xlo = __double2int_rn(((double)xl - f.xc) * f.sx);
@@ -1908,11 +1915,15 @@ __global__ void __launch_bounds__(T) k_direct(const DirectArgs A)
         // above every pair's slope; float sets leave steeper ones to the bound below
         const long long kmax = F ? F_KMAX : ((long long)yr + 1) << 32;
 
-        // Float sets: w at a slope differs by at most (1 + |s|) steps from w of the
-        // grid points.  An upper bound is raised by that much, and an interval is
+        // Float sets: w at a slope differs by at most (1 + |s|) steps and the rounding
+        // of its doubles from w of the grid points.  An upper bound is raised by that much, and an interval is
         // tested against the upper bound raised once more.
         auto grid_key = [&](double s) { return (long long)floor(s * fs.ratio * (double)(1LL << F_YS)); };
-        auto grid_err = [](long long K) { return F ? (1LL << F_YS) + (K < 0 ? -K : K) + 4 : 0LL; };
+        auto grid_err = [&](long long K) {
+            if (!F) return 0LL;
+            const long long k = K < 0 ? -K : K;
+            return (1LL << F_YS) + k + 4 + (long long)(fs.rx * (double)k + fs.ry);
+        };
 
         // ---------------------------------------------------------- sampled slopes (the same in every CTA)
         {

@@ -97,3 +97,18 @@ def test_float_shared_slopes_finish(D, kind, n):
     """Pairs that share a slope are listed once (a leaf of one slope key overflowed its list: 403 phases, given up)."""
     done, _, c = D.f32(*points(kind, n, n))
     assert done and c["phases"] <= 24, c
+
+
+@pytest.mark.parametrize("offset", [0.0, 1e2, 1e4, 1e5, 1e6, 1e7])
+def test_float_far_from_the_origin(D, offset):
+    """A common offset of up to the float's precision: the double projections round by up to a few steps of the grid
+    that prunes, which no interval may be dropped for."""
+    rng = np.random.default_rng(int(offset) + 1)
+    finished = 0
+    for trial in range(12):
+        n = int(rng.integers(24, 120))
+        x, y = offset + rng.normal(size=n), rng.normal(size=n) + (offset if trial % 2 else 0)
+        x, y = x.astype(np.float32), y.astype(np.float32)
+        for h in (0, int(0.8 * n)):
+            finished += check_float(D, x, y, h)[0]
+    assert finished or offset > 1e6
