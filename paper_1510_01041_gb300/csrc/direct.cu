@@ -71,6 +71,8 @@ constexpr int EV_F = 8;                    // children of a run of slopes
 constexpr int TABLE = 2048;                // slots of a CTA's slope table
 constexpr float LEAF_FRACTIONS = 32.0f;      // an interval with this few possible slopes is a leaf
 constexpr float FRACTIONS = 1000.0f;         // expected fractions of a leaf up to which they are tried one by one
+constexpr int REGROW = 3;                    // .. times that leaves are cut instead when they hold more
+constexpr float LIST_HOPE = 4.0f;            // .. leaves are listed together up to so many lists of expected slopes
 constexpr int CELLS_MAX = 8192;             // cells of the pair search
 constexpr float DENSE = 16384.0f;            // candidates up to which a leaf's pairs are searched in the cells ..
 constexpr float DENSE_PER_POINT = 64.0f;     // .. and so many more for each point (ordinary sets: at most 30 a point)
@@ -80,7 +82,7 @@ constexpr int DEPTH_MAX = 28;              // levels: an interval has fewer than
 // A float set is left to the sweep beyond these (ordinary sets: at most 13 phases, 1 cut, 130 slopes scored).
 constexpr int F_SCORES = 256;              // slopes scored
 constexpr int F_PHASES = 48;
-constexpr int F_CUTS = 3;                  // lists that did not hold their leaves' slopes
+constexpr int F_CUTS = 6;                  // lists that did not hold their leaves' slopes
 constexpr int PHASES_MAX = 1 << 20;        // phases of one fit before it is reported as failed
 constexpr int RUN_MIN = 12;                // slopes a CTA scores from which it keeps the points sorted between them
 constexpr int EXCHANGES = 16;              // passes that repair their order, else they are sorted again
@@ -2223,7 +2225,7 @@ __global__ void __launch_bounds__(T) k_direct(const DirectArgs A)
                         held += F ? S.leaf[l].est * gain : leaf_slopes(S.leaf[l], gain, xr, yr);
                     if (F && (over == 2 || (over && (++cuts_more > F_CUTS || (lfn == 1 && S.leaf[lf0].b - S.leaf[lf0].a == 1)))))
                         err = 1;   // more slopes or candidates than the sweep is worth
-                    if (over) gain = fminf(1.0f, 4.0f * gain);
+                    if (over == 1 && lfn == 1) gain = fminf(64.0f, 4.0f * gain);
                     else if (8.0f * (float)nn < held) gain = fmaxf(1.0f / 4096, 0.25f * gain);
                 }
                 if constexpr (!F) {
@@ -2325,19 +2327,21 @@ __global__ void __launch_bounds__(T) k_direct(const DirectArgs A)
                     }
                 } else if (over == 2) {
                     P = 0;
-                } else if (lfn > 1 && regrown < (F ? 8 : 2) && lfn <= PM && lfn == nleaf) {
-                    // their expected pairs were too low: cut them once more
-                    for (int j = threadIdx.x; j < lfn; j += T) {
-                        DNode nd = S.leaf[j];
+                } else if (regrown < REGROW && nleaf - lf0 > 1 && nleaf - lf0 <= PM) {
+                    // more slopes than hoped: the leaves are cut and tested once more
+                    const int left = nleaf - lf0;
+                    for (int j = threadIdx.x; j < left; j += T) {
+                        DNode nd = S.leaf[lf0 + j];
                         nd.force = 1;
                         S.work[cur][j] = nd;
                     }
                     ++regrown;
-                    P = -lfn;
-                    nleaf = 0;
+                    P = -left;
+                    lf0 = nleaf = 0;
                     flush = false;
                 } else if (lfn > 1) {
-                    lfn = lcap = max(1, lfn / 4);
+                    // fewer of them: as many as would have fitted
+                    lfn = lcap = max(1, min(lfn / 2, (int)(0.6f * (float)lfn * (float)sh.HC / (float)max(nn, 1))));
                     P = 0;
                 } else {
                     // one leaf with too many slopes: more intervals of it, the other leaves wait on the stack
@@ -2481,7 +2485,7 @@ __global__ void __launch_bounds__(T) k_direct(const DirectArgs A)
                     int l = 0;
                     for (; l < lfn; ++l) {
                         held += F ? fmaxf(S.leaf[lf0 + l].est * gain, 1.0f) : leaf_slopes(S.leaf[lf0 + l], gain, xr, yr);
-                        if (l > 0 && held > 0.75f * (float)sh.HC) break;
+                        if (l > 0 && held > LIST_HOPE * (float)sh.HC) break;
                     }
                     lfn = max(1, l);
                 }
