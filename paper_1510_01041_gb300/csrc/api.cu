@@ -168,11 +168,11 @@ int run_fit(const void *x, const void *y, int n, int h, int dtype, const lms_opt
             cudaStream_t st, void *ws_in, const Choice &c)
 {
     cudaGetLastError();
-    if (c.direct && dtype == LMS_I16)
-        return launch_direct((const short *)x, (const short *)y, n, h, c.algo, nullptr, out, ws_in, st) ==
-                       cudaSuccess
-                   ? LMS_OK
-                   : LMS_ERR_CUDA;
+    if (c.direct && dtype == LMS_I16) {
+        if (launch_direct((const short *)x, (const short *)y, n, h, c.algo, nullptr, out, ws_in, st) == cudaSuccess)
+            return LMS_OK;
+        cudaGetLastError();   // no room for its cluster: the sweep
+    }
     if (c.algo == LMS_ALGO_PLAIN) {
         Cand *cands = static_cast<Cand *>(ws_in);
         if (launch_plain((const short *)x, (const short *)y, n, h, cands, c.plain_warps, st) != cudaSuccess)
@@ -195,10 +195,11 @@ int run_fit(const void *x, const void *y, int n, int h, int dtype, const lms_opt
         // the one-kernel branch-and-bound first, on the same workspace; the
         // sweep's kernels return at once when it has written the record
         int *done = reinterpret_cast<int *>(static_cast<unsigned char *>(ws_in) + c.bytes - 64);
-        if (launch_direct_f32((const float *)x, (const float *)y, n, h, LMS_ALGO_SWEEP, out, done, ws_in, st) !=
+        if (launch_direct_f32((const float *)x, (const float *)y, n, h, LMS_ALGO_SWEEP, out, done, ws_in, st) ==
             cudaSuccess)
-            return LMS_ERR_CUDA;
-        p.skip = done;
+            p.skip = done;
+        else
+            cudaGetLastError();   // no room for its cluster
     }
     if (dtype == LMS_F32)
         return launch_sweep_f32_fit(p, (const float *)x, (const float *)y,
@@ -266,10 +267,9 @@ int fit_bnb_after(const void *x, const void *y, int64_t n, int64_t h, const floa
         direct_bytes((int)n) <= c.bytes) {
         if (pred_ready && cudaStreamWaitEvent(st, pred_ready, 0) != cudaSuccess) return LMS_ERR_CUDA;
         cudaGetLastError();
-        return launch_direct((const short *)x, (const short *)y, (int)n, (int)h, LMS_ALGO_BNB, seed_slope, out, ws,
-                             st) == cudaSuccess
-                   ? LMS_OK
-                   : LMS_ERR_CUDA;
+        if (launch_direct((const short *)x, (const short *)y, (int)n, (int)h, LMS_ALGO_BNB, seed_slope, out, ws, st) ==
+            cudaSuccess)
+            return LMS_OK;   // (else no room for its cluster)
     }
     SweepPlan p = c.sweep;
     sweep_plan_carve(p, ws);

@@ -317,12 +317,11 @@ int lms_batch_plan_create_ex(const int64_t *offsets_host, int64_t B, const int32
         p->hval[i] = h;
     }
     // classes
-    std::vector<int> members[3], direct;
+    std::vector<int> members[3], direct, rest;
     for (int64_t i = 0; i < B; ++i) {
         const int64_t n = offsets_host[i + 1] - offsets_host[i];
-        if (n <= p->plain_max && (n < BATCH_DIRECT_MIN || !direct_ok((int)n, p->hval[i]))) members[n <= 64 ? 0 : (n <= 128 ? 1 : 2)].push_back((int)i);
-        else if (n <= DIRECT_BATCH_MAX && direct_ok((int)n, p->hval[i])) direct.push_back((int)i);
-        else p->sweep_sets.push_back((int)i);
+        if (n >= BATCH_DIRECT_MIN && n <= DIRECT_BATCH_MAX && direct_ok((int)n, p->hval[i])) direct.push_back((int)i);
+        else rest.push_back((int)i);
     }
     std::sort(direct.begin(), direct.end(), [&](int a, int b) {
         return offsets_host[a + 1] - offsets_host[a] > offsets_host[b + 1] - offsets_host[b];
@@ -331,7 +330,16 @@ int lms_batch_plan_create_ex(const int64_t *offsets_host, int64_t B, const int32
         p->ndirect = (int)direct.size();
         p->direct_nmax = (int)(offsets_host[direct[0] + 1] - offsets_host[direct[0]]);
         p->direct_teams = direct_batch_teams(p->ndirect, p->direct_nmax, sms);
-        if (p->direct_teams < 1) { delete p; return LMS_ERR_CUDA; }
+        if (p->direct_teams < 1) {   // a device without room for its CTAs
+            p->ndirect = 0;
+            rest.insert(rest.end(), direct.begin(), direct.end());
+            direct.clear();
+        }
+    }
+    for (const int i : rest) {
+        const int64_t n = offsets_host[i + 1] - offsets_host[i];
+        if (n <= p->plain_max) members[n <= 64 ? 0 : (n <= 128 ? 1 : 2)].push_back(i);
+        else p->sweep_sets.push_back(i);
     }
     size_t bytes = a256(sizeof(int) * B) + a256(sizeof(int) * direct.size()) +
                    (p->ndirect ? direct_batch_bytes(p->direct_teams, p->direct_nmax) : 0);

@@ -45,6 +45,9 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <map>
+#include <mutex>
+#include <tuple>
 #include <type_traits>
 
 #include "common.cuh"
@@ -2622,6 +2625,28 @@ Single float_single_of(int n)
     return s;
 }
 
+// Whether the current device can hold one cluster of this kernel (16 CTAs are
+// more than every device or partition of one grants), asked once per device,
+// kernel and size of shared memory.
+bool cluster_fits(const void *kern, const cudaLaunchConfig_t &cfg)
+{
+    static std::mutex mu;
+    static std::map<std::tuple<int, const void *, size_t>, bool> known;
+    int dev;
+    if (cudaGetDevice(&dev) != cudaSuccess) return false;
+    std::lock_guard<std::mutex> lock(mu);
+    const auto key = std::make_tuple(dev, kern, cfg.dynamicSmemBytes);
+    const auto it = known.find(key);
+    if (it != known.end()) return it->second;
+    int clusters = 0;
+    const bool fits = cudaOccupancyMaxActiveClusters(&clusters, kern, &cfg) == cudaSuccess && clusters > 0;
+    if (known.size() > 4096) known.clear();
+    known[key] = fits;
+    return fits;
+}
+
+// An error (not launched) also where the device cannot hold the cluster: the
+// caller then takes the path of many kernels.
 template <class SH>
 cudaError_t launch_cluster(const DirectArgs &a, size_t smem, cudaStream_t st)
 {
@@ -2641,6 +2666,8 @@ cudaError_t launch_cluster(const DirectArgs &a, size_t smem, cudaStream_t st)
     at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
+    if (!cluster_fits(reinterpret_cast<const void *>(kern), cfg)) return cudaErrorLaunchOutOfResources;
+    StageTimer _t(STAGE_DIRECT, st);
     return cudaLaunchKernelEx(&cfg, kern, a);
 }
 
@@ -2674,7 +2701,6 @@ cudaError_t launch_direct(const short *x, const short *y, int n, int h, int algo
     a.out = out;
     a.mem = static_cast<unsigned char *>(mem);
     a.shape = s.shape;
-    StageTimer _t(STAGE_DIRECT, st);
     if (s.variant == 0) return launch_cluster<Small>(a, s.smem, st);
     if (s.variant == 1) return launch_cluster<Mid>(a, s.smem, st);
     return launch_cluster<Large>(a, s.smem, st);
@@ -2701,7 +2727,6 @@ cudaError_t launch_direct_f32(const float *x, const float *y, int n, int h, int 
     a.shape = s.shape;
     cudaError_t e = cudaMemsetAsync(done, 0, sizeof(int), st);
     if (e != cudaSuccess) return e;
-    StageTimer _t(STAGE_DIRECT, st);
     return s.variant == 0 ? launch_cluster<FloatSmall>(a, s.smem, st) : launch_cluster<FloatMid>(a, s.smem, st);
 }
 

@@ -30,6 +30,7 @@ std::map<void *, size_t> blocks;
 std::map<std::string, long long> knobs = {
     {"clusters", 8},         // clusters that can be resident
     {"refuse_clusters", 0},  // launches of a cluster fail
+    {"no_blocks", 0},        // no CTA can be resident
     {"capturing", 0},        // streams are being captured
     {"sms", 152}};
 long long frees = 0;
@@ -140,7 +141,7 @@ cudaError_t cudaOccupancyMaxActiveBlocksPerMultiprocessorWithFlags(int *n, const
     std::lock_guard<std::mutex> lock(mu);
     *n = 0;
     if (smem > kernels[f].limit) return done(cudaErrorInvalidValue);
-    *n = smem ? (int)(227 * 1024 / smem) : 8;
+    *n = knobs["no_blocks"] ? 0 : smem ? (int)(227 * 1024 / smem) : 8;
     return cudaSuccess;
 }
 cudaError_t cudaOccupancyMaxActiveClusters(int *n, const void *, const cudaLaunchConfig_t *)

@@ -79,3 +79,32 @@ def test_shared_memory_limits_are_only_raised(H):
             assert v >= sizes.get(k, 0), (n, k)
         sizes.update(limits)
     assert max(sizes.values()) > 48 * 1024
+
+
+# ---------------------------------------------------------------- routes
+def route(names):
+    """What a call's kernels are: the one kernel, the sweep's, the staged branch-and-bound's, the plain ones."""
+    parts = {"one": "k_direct", "sweep": "k_sweep", "staged": "k_node_lb", "plain": "k_plain"}
+    return {k for k, part in parts.items() if any(part in n for n in names)}
+
+
+@pytest.mark.parametrize("knob,value", [("clusters", 0), ("refuse_clusters", 1)])
+def test_no_room_for_the_cluster(H, knob, value):
+    """A device that cannot hold the one kernel's cluster, or a launch it refuses: the fits take the paths of many
+    kernels."""
+    H.set(knob, value)
+    for call, want in ((lambda: H.fit(2048), {"sweep"}), (lambda: H.fit(8192, host=True), {"sweep"}),
+                       (lambda: H.fit(2048, dtype=F32), {"sweep"}), (lambda: H.fit_bnb(2048), {"staged", "sweep"}),
+                       (lambda: H.fit_bnb(65536), {"staged", "sweep"})):
+        assert call() == 0
+        assert route(H.kernels()) == want
+    H.set("clusters", 8)
+    H.set("refuse_clusters", 0)
+
+
+def test_batch_without_room_for_the_one_kernel(H):
+    H.set("no_blocks", 1)
+    rc, plan, off = H.plan([64, 200, 300, 2000])
+    assert rc == 0 and H.fit_batched(plan, off) == 0
+    assert route(H.kernels()) == {"plain", "staged", "sweep"}
+    H.set("no_blocks", 0)
