@@ -140,6 +140,8 @@ int choose(int n, int h, int dtype, const lms_options *opt, int dev, Choice &c)
     }
     c.bytes += 256;   // result staging for host-pointer calls, and the flag of a float fit
     if (dtype == LMS_F32) c.direct = algo_req == LMS_ALGO_AUTO && direct_f32_ok(n, h);
+    // sweepers and buckets are the sweep's: a call that sets them gets the sweep
+    if (opt && (opt->sweepers || opt->buckets)) c.direct = false;
     // the one kernel's scratch lies in the same workspace (it needs far less: 2.8 MB of 42 at n = 2048)
     if (c.direct && (dtype == LMS_F32 ? direct_f32_bytes(n) : direct_bytes(n)) + 256 > c.bytes) c.direct = false;
     return LMS_OK;

@@ -316,11 +316,15 @@ int lms_batch_plan_create_ex(const int64_t *offsets_host, int64_t B, const int32
         if (h < 1 || h > n) { delete p; return LMS_ERR_ARG; }
         p->hval[i] = h;
     }
-    // classes
+    // classes.  A given plain_max_n or bnb_min_n is kept to: the plain kernel up
+    // to the one, a branch-and-bound only from the other on.  Left to the library
+    // (0), sets from BATCH_DIRECT_MIN points on take the one kernel.
     std::vector<int> members[3], direct, rest;
     for (int64_t i = 0; i < B; ++i) {
         const int64_t n = offsets_host[i + 1] - offsets_host[i];
-        if (n >= BATCH_DIRECT_MIN && n <= DIRECT_BATCH_MAX && direct_ok((int)n, p->hval[i])) direct.push_back((int)i);
+        const bool bnb = bnb_min_n == 0 || n >= p->bnb_min;
+        const bool one = n >= BATCH_DIRECT_MIN && n <= DIRECT_BATCH_MAX && bnb && direct_ok((int)n, p->hval[i]);
+        if (one && (n > p->plain_max || (plain_max_n <= 0 && bnb_min_n == 0))) direct.push_back((int)i);
         else rest.push_back((int)i);
     }
     std::sort(direct.begin(), direct.end(), [&](int a, int b) {

@@ -102,6 +102,30 @@ def test_no_room_for_the_cluster(H, knob, value):
     H.set("refuse_clusters", 0)
 
 
+def test_sweep_options_take_the_sweep(H):
+    assert H.fit(2048) == 0 and route(H.kernels()) == {"one"}
+    for opt in ({"sweepers": 100}, {"buckets": 64}):
+        assert H.fit(2048, **opt) == 0 and route(H.kernels()) == {"sweep"}
+        assert H.fit(2048, dtype=F32, **opt) == 0 and route(H.kernels()) == {"sweep"}
+
+
+# default: plain, then the one kernel up to 4096 points, staged above; options are kept to
+@pytest.mark.parametrize("options,want", [
+    ({}, {64: "plain", 256: "one", 400: "one", 512: "one", 4096: "one", 4097: "staged"}),
+    ({"plain_max_n": 128}, {64: "plain", 128: "plain", 256: "one", 512: "one", 4097: "staged"}),
+    ({"plain_max_n": 256}, {256: "plain", 400: "one", 4096: "one"}),
+    ({"bnb_min_n": -1}, {256: "plain", 257: "sweep", 4096: "sweep", 4097: "sweep"}),
+    ({"bnb_min_n": 512}, {256: "plain", 400: "sweep", 511: "sweep", 512: "one", 4097: "staged"}),
+    ({"plain_max_n": 64, "bnb_min_n": 600}, {64: "plain", 100: "sweep", 599: "sweep", 600: "one", 5000: "staged"})])
+def test_batch_options_choose_the_path(H, options, want):
+    for n, path in want.items():
+        rc, plan, off = H.plan([n], **options)
+        assert rc == 0 and H.fit_batched(plan, off) == 0
+        got = route(H.kernels())
+        assert got == ({"staged", "sweep"} if path == "staged" else {path}), (n, options)
+        H.lib.lms_batch_plan_destroy(plan)
+
+
 def test_batch_without_room_for_the_one_kernel(H):
     H.set("no_blocks", 1)
     rc, plan, off = H.plan([64, 200, 300, 2000])
