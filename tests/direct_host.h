@@ -1,4 +1,4 @@
-// What a host build of the one-kernel branch-and-bound (direct.cu) needs of
+// What a host build of the one-kernel branch-and-bound (direct.cuh) needs of
 // CUDA: one thread runs a whole team (T = G = 1, one CTA), so barriers do
 // nothing and a warp has one lane.  Included by the file direct_host.py makes.
 #pragma once

@@ -1,4 +1,4 @@
-"""The one-kernel branch-and-bound (direct.cu) built for the host: the
+"""The one-kernel branch-and-bound (direct.cuh) built for the host: the
 kernel's own code run by one thread (direct_host.h), with counters of its
 phases, on sets of any form, without a GPU.  Barriers and races are not
 covered; answers, give-ups, loops and the amount of work are."""
@@ -56,7 +56,7 @@ def source():
     common = open(os.path.join(CSRC, "common.cuh")).read()
     a, b = common.index("// Ascending bitonic sort of P = IPT"), common.index("// A range's start order (global")
     common = common[:a] + common[b:]          # its sorting helpers: direct_host.h has them
-    direct = open(os.path.join(CSRC, "direct.cu")).read()
+    direct = open(os.path.join(CSRC, "direct.cuh")).read()
     direct = direct[:direct.index("// ------------------------------------------------------------------ host\n")]
     for name, body in (("unsigned cluster_ctas()", "return 1;"), ("unsigned cluster_rank()", "return 0;"),
                        ("unsigned smem_size()", "return sizeof(dsm);"), ("void cluster_meet()", ""),
@@ -68,7 +68,7 @@ def source():
     text = common + direct
     text = re.sub(r"#include.*\n|#pragma once\n", "", text)
     return ('#include "direct_host.h"\n#include "lms.h"\n'
-            "static unsigned char dsm[1 << 20] __attribute__((aligned(16)));\n" + text + "}\n}\nusing namespace lms;\n"
+            "static unsigned char dsm[1 << 20] __attribute__((aligned(16)));\n" + text + "}\n}\nusing namespace lms;\nusing namespace lms::direct;\n"
             + ENTRY)
 
 
