@@ -86,7 +86,12 @@ Single float_single_of(int n)
 // 9.2 - 10.3), each scored by a sort.
 bool direct_f32_ok(int n, int h) { return n >= 16 && n <= 4096 && (long long)h * 4 >= n; }
 
-bool direct_ok(int n, int h) { return n >= 2 && n <= 65536 && (long long)h * 8 >= n; }
+// A small order statistic leaves many intervals alive.  Against the paths of
+// many kernels, ordinary sets (lines, random points, curves; median and largest
+// ratio of times): h = n / 3: batches of 4096-point sets 0.28 and 0.54, single
+// fits at 2048 points 0.58 and 1.04; h = n / 4: 0.35 and 15, 0.63 and 1.03;
+// h = n / 8: 0.38 and 25, 0.62 and 1.64.
+bool direct_ok(int n, int h) { return n >= 2 && n <= 65536 && (long long)h * 3 >= n; }
 
 size_t direct_bytes(int n) { return (size_t)d_up(team_bytes(single_of(n).shape)); }
 
