@@ -21,7 +21,12 @@ namespace lms {
 namespace {
 
 constexpr int CHUNK = 64;   // slopes per work item of the plain kernel
-constexpr int BATCH_DIRECT_MIN = 65;    // sets from this size take one CTA of the one-kernel branch-and-bound
+// Sets from this size take one CTA of the one-kernel branch-and-bound, and the
+// per-slope kernel when that takes long.  (Median order statistic, ordinary
+// sets, against the per-slope kernel alone: 65 points 1.05, 80 0.73, 97 0.59,
+// 128 0.36, 256 0.07 of the time.)
+constexpr int BATCH_DIRECT_MIN = 97;
+constexpr int PLAIN_CLASS_MAX = 256;    // points of the largest plain class
 constexpr int BATCH_BNB_MIN_N = 512;   // default size from which a set takes the branch-and-bound
 
 template <typename K>
@@ -76,14 +81,15 @@ __device__ __forceinline__ void wsort(K (&v)[E], int lane)
 }
 
 // One warp per chunk of at most CHUNK consecutive slopes of one set.
-// chunk_pre[i] = chunks before class-set i; sets[i] = global set index.
+// chunk_pre[i] = chunks before class-set i; sets[i] = global set index.  Sets
+// that the one kernel has fitted (done, by global set index) are passed over.
 template <int E>
 __global__ void __launch_bounds__(256) k_plain_batched(const short *__restrict__ x, const short *__restrict__ y,
                                                        const long long *__restrict__ off,
                                                        const int *__restrict__ hvec,
                                                        const int *__restrict__ sets, int nsets,
                                                        const long long *__restrict__ chunk_pre,
-                                                       Cand *__restrict__ outc)
+                                                       const int *__restrict__ done, Cand *__restrict__ outc)
 {
     __shared__ long long s_buf[8][32 * E];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -93,6 +99,7 @@ __global__ void __launch_bounds__(256) k_plain_batched(const short *__restrict__
         int lo = 0, hi = nsets;
         while (hi - lo > 1) { const int mid = (lo + hi) >> 1; if (chunk_pre[mid] <= c) lo = mid; else hi = mid; }
         const int si = lo;
+        if (done[sets[si]]) continue;
         const long long base = off[sets[si]];
         const int n = (int)(off[sets[si] + 1] - base);
         const int h = hvec[sets[si]];
@@ -169,12 +176,12 @@ __global__ void __launch_bounds__(256) k_plain_batched(const short *__restrict__
 __global__ void k_plain_batched_reduce(const short *__restrict__ x, const short *__restrict__ y,
                                        const long long *__restrict__ off, const int *__restrict__ hvec,
                                        const int *__restrict__ sets, int nsets,
-                                       const long long *__restrict__ chunk_pre, const Cand *__restrict__ outc,
-                                       Cand *__restrict__ best_out)
+                                       const long long *__restrict__ chunk_pre, const int *__restrict__ done,
+                                       const Cand *__restrict__ outc, Cand *__restrict__ best_out)
 {
     const int lane = threadIdx.x & 31;
     const int si = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (si >= nsets) return;
+    if (si >= nsets || done[sets[si]]) return;
     Cand best = cand_empty();
     for (long long c = chunk_pre[si] + lane; c < chunk_pre[si + 1]; c += 32)
         if (cand_better(outc[c], best)) best = outc[c];
@@ -216,14 +223,15 @@ __device__ __forceinline__ long long gcd_ll(long long a, long long b)
 }
 
 // Translate per-set winners into lms_result records at their set indices.
-__global__ void k_batched_finish(const Cand *__restrict__ best, const int *__restrict__ sets, int nsets,
+__global__ void k_batched_finish(const Cand *__restrict__ best, const long long *__restrict__ off,
+                                 const int *__restrict__ sets, int nsets, const int *__restrict__ done, int plain_max,
                                  lms_result *__restrict__ out)
 {
     const int si = blockIdx.x * blockDim.x + threadIdx.x;
-    if (si >= nsets) return;
+    if (si >= nsets || done[sets[si]]) return;
     const Cand b = best[si];
     lms_result r;
-    r.algorithm = LMS_ALGO_PLAIN;
+    r.algorithm = off[sets[si] + 1] - off[sets[si]] <= plain_max ? LMS_ALGO_PLAIN : LMS_ALGO_SWEEP;
     const long long dx = b.dx, dy = b.dy;
     long long g = gcd_ll(dy < 0 ? -dy : dy, dx);
     if (g <= 0) g = 1;
@@ -262,6 +270,7 @@ struct lms_batch_plan {
         Cand *best = nullptr;           // device
     } cls[3];
     int *hvec = nullptr;                // device, per set
+    int *set_done = nullptr;            // device, per set: fitted by the one kernel (0 for those of the plain classes alone)
     // sets of the one-kernel branch-and-bound (direct.cu), largest first
     int ndirect = 0, direct_teams = 0, direct_nmax = 0;
     int *direct_sets = nullptr;         // device
@@ -302,7 +311,7 @@ int lms_batch_plan_create_ex(const int64_t *offsets_host, int64_t B, const int32
     int sms = 1;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, p->dev);
     p->B = B;
-    p->plain_max = plain_max_n > 0 ? std::min(plain_max_n, 256) : 256;
+    p->plain_max = plain_max_n > 0 ? std::min(plain_max_n, PLAIN_CLASS_MAX) : PLAIN_CLASS_MAX;
     // sets from this size on take the branch-and-bound (its fixed cost, a few
     // hundred microseconds of seeds and bounds, pays off once the sweep of every
     // slope costs more); negative: never
@@ -345,7 +354,12 @@ int lms_batch_plan_create_ex(const int64_t *offsets_host, int64_t B, const int32
         if (n <= p->plain_max) members[n <= 64 ? 0 : (n <= 128 ? 1 : 2)].push_back(i);
         else p->sweep_sets.push_back(i);
     }
-    size_t bytes = a256(sizeof(int) * B) + a256(sizeof(int) * direct.size()) +
+    // the one kernel may leave its small sets to the plain classes
+    for (const int i : direct) {
+        const int64_t n = offsets_host[i + 1] - offsets_host[i];
+        if (n <= PLAIN_CLASS_MAX) members[n <= 128 ? 1 : 2].push_back(i);
+    }
+    size_t bytes = 2 * a256(sizeof(int) * B) + a256(sizeof(int) * direct.size()) +
                    (p->ndirect ? direct_batch_bytes(p->direct_teams, p->direct_nmax) : 0);
     std::vector<std::vector<long long>> pres(3);
     for (int c = 0; c < 3; ++c) {
@@ -368,6 +382,8 @@ int lms_batch_plan_create_ex(const int64_t *offsets_host, int64_t B, const int32
     auto take = [&](size_t b) { void *r = q; q += a256(b); return r; };
     p->hvec = (int *)take(sizeof(int) * B);
     cudaMemcpy(p->hvec, p->hval.data(), sizeof(int) * B, cudaMemcpyHostToDevice);
+    p->set_done = (int *)take(sizeof(int) * B);
+    cudaMemset(p->set_done, 0, sizeof(int) * B);
     if (p->ndirect) {
         p->direct_sets = (int *)take(sizeof(int) * direct.size());
         cudaMemcpy(p->direct_sets, direct.data(), sizeof(int) * direct.size(), cudaMemcpyHostToDevice);
@@ -456,7 +472,8 @@ int lms_fit_batched(lms_batch_plan *p, const void *xv, const void *yv, const int
     bool failed = false;
     if (p->ndirect)
         failed = launch_direct_batch(x, y, off, p->hvec, p->direct_sets, p->ndirect, p->direct_nmax, p->direct_teams,
-                                     p->plain_max, p->bnb_min, out, p->direct_mem, st) != cudaSuccess;
+                                     p->plain_max, p->bnb_min, p->set_done, PLAIN_CLASS_MAX, out, p->direct_mem, st) !=
+                 cudaSuccess;
     for (int c = 0; c < 3; ++c) {
         auto &C = p->cls[c];
         if (C.nsets == 0) continue;
@@ -466,19 +483,20 @@ int lms_fit_batched(lms_batch_plan *p, const void *xv, const void *yv, const int
         if (C.nchunks > 0) {
             StageTimer _t(STAGE_PLAIN, st);
             switch (C.E) {
-                case 2: k_plain_batched<2><<<(int)std::max(1LL, blocks), 256, 0, st>>>(x, y, off, p->hvec, C.sets, C.nsets, C.chunk_pre, C.outc); break;
-                case 4: k_plain_batched<4><<<(int)std::max(1LL, blocks), 256, 0, st>>>(x, y, off, p->hvec, C.sets, C.nsets, C.chunk_pre, C.outc); break;
-                default: k_plain_batched<8><<<(int)std::max(1LL, blocks), 256, 0, st>>>(x, y, off, p->hvec, C.sets, C.nsets, C.chunk_pre, C.outc); break;
+                case 2: k_plain_batched<2><<<(int)std::max(1LL, blocks), 256, 0, st>>>(x, y, off, p->hvec, C.sets, C.nsets, C.chunk_pre, p->set_done, C.outc); break;
+                case 4: k_plain_batched<4><<<(int)std::max(1LL, blocks), 256, 0, st>>>(x, y, off, p->hvec, C.sets, C.nsets, C.chunk_pre, p->set_done, C.outc); break;
+                default: k_plain_batched<8><<<(int)std::max(1LL, blocks), 256, 0, st>>>(x, y, off, p->hvec, C.sets, C.nsets, C.chunk_pre, p->set_done, C.outc); break;
             }
         }
         {
             StageTimer _t(STAGE_ARGMIN, st);
             k_plain_batched_reduce<<<(C.nsets + 7) / 8, 256, 0, st>>>(x, y, off, p->hvec, C.sets, C.nsets, C.chunk_pre,
-                                                                      C.outc, C.best);
+                                                                      p->set_done, C.outc, C.best);
         }
         {
             StageTimer _t(STAGE_ARGMIN, st);
-            k_batched_finish<<<(C.nsets + 127) / 128, 128, 0, st>>>(C.best, C.sets, C.nsets, out);
+            k_batched_finish<<<(C.nsets + 127) / 128, 128, 0, st>>>(C.best, off, C.sets, C.nsets, p->set_done, p->plain_max,
+                                                                    out);
         }
     }
     // sweep sets on their streams

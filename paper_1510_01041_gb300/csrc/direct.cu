@@ -157,8 +157,8 @@ size_t direct_batch_bytes(int nteams, int nmax)
 }
 
 cudaError_t launch_direct_batch(const short *x, const short *y, const long long *off, const int *hvec, const int *sets,
-                                int nsets, int nmax, int nteams, int plain_max, int bnb_min, lms_result *out,
-                                void *mem, cudaStream_t st)
+                                int nsets, int nmax, int nteams, int plain_max, int bnb_min, int *set_done,
+                                int small_max, lms_result *out, void *mem, cudaStream_t st)
 {
     DirectArgs a = {};
     a.x = x;
@@ -170,6 +170,8 @@ cudaError_t launch_direct_batch(const short *x, const short *y, const long long 
     a.algo = LMS_ALGO_SWEEP;
     a.plain_max = plain_max;
     a.bnb_min = bnb_min;
+    a.set_done = set_done;
+    a.small_max = small_max;
     a.out = out;
     a.next = static_cast<int *>(mem);
     a.mem = static_cast<unsigned char *>(mem) + 256;

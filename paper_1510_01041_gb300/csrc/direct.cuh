@@ -88,6 +88,10 @@ constexpr int F_CUTS = 6;                  // lists that did not hold their leav
 constexpr int PHASES_MAX = 1 << 20;        // phases of one fit before it is reported as failed
 constexpr int RUN_MIN = 12;                // slopes a CTA scores from which it keeps the points sorted between them
 constexpr int EXCHANGES = 16;              // passes that repair their order, else they are sorted again
+// A small set of a batch is left to the per-slope kernel beyond these (ordinary
+// sets up to 256 points: at most 16 phases and 12 slopes scored).
+constexpr int SMALL_PHASES = 20;
+constexpr int SMALL_SCORES = 64;
 constexpr int EV_DEPTH = 6;                // levels of a run of at most EV_F^EV_DEPTH slopes
 
 struct DNode {
@@ -1688,6 +1692,8 @@ struct DirectArgs {
     lms_result *out;
     unsigned char *mem;           // teams' memory
     int *next;                    // next set (several sets)
+    int *set_done;                // per set (or null): 0 when a set of at most small_max points is left to another kernel
+    int small_max;
     int n, h, nsets;
     int algo, plain_max, bnb_min;   // reported path: PLAIN up to plain_max points, BNB from bnb_min on, else algo
     TeamShape shape;
@@ -1889,6 +1895,8 @@ __global__ void __launch_bounds__(T) k_direct(const DirectArgs A)
             st->nlist[0] = st->nlist[1] = st->over[0] = st->over[1] = 0;
         }
         team_sync();
+        [[maybe_unused]] const bool brief = !F && A.set_done && n <= A.small_max;
+        const int phases = F ? F_PHASES : brief ? SMALL_PHASES : PHASES_MAX;
         const int algo = n <= A.plain_max ? LMS_ALGO_PLAIN : n >= A.bnb_min ? LMS_ALGO_BNB : A.algo;
         if constexpr (!F) {
         if (S.bx.xlo == S.bx.xhi) {
@@ -1896,7 +1904,10 @@ __global__ void __launch_bounds__(T) k_direct(const DirectArgs A)
             if (rank == 0) {
                 Cand c = score<T>(pts, n, h, 0, 1, S.bx, wk, wk_bytes, gsort, S.red);
                 c.i = c.j = -1;
-                if (threadIdx.x == 0) write_result(A.out + set, c, algo, 0);
+                if (threadIdx.x == 0) {
+                    write_result(A.out + set, c, algo, 0);
+                    if (brief) A.set_done[set] = 1;
+                }
             }
             team_sync();
             continue;
@@ -2363,7 +2374,7 @@ __global__ void __launch_bounds__(T) k_direct(const DirectArgs A)
                 }
                 team_sync();
                 if (over && P == 0) {
-                    if (phase > (F ? F_PHASES : PHASES_MAX)) err = 1;
+                    if (phase > phases) err = 1;
                     mode = err ? M_DONE : M_PAIRS;
                     continue;
                 }
@@ -2458,7 +2469,8 @@ __global__ void __launch_bounds__(T) k_direct(const DirectArgs A)
             }
             // ---------------------------------------------------- the next phase
             const bool was_tree = mode == M_TREE;
-            if (err || phase > (F ? F_PHASES : PHASES_MAX)) {
+            if (!F && nx > 0) scored += nx;
+            if (err || phase > phases || (brief && scored > SMALL_SCORES)) {
                 err = 1;
                 mode = M_DONE;
             } else if (nx > 0) {
@@ -2534,7 +2546,11 @@ __global__ void __launch_bounds__(T) k_direct(const DirectArgs A)
                 *A.done = 1;
             }
         } else {
-            if (rank == 0 && threadIdx.x == 0) write_result(A.out + set, best, algo, err | __ldcg(&st->bad));
+            if (rank == 0 && threadIdx.x == 0) {
+                const int bad = err | __ldcg(&st->bad);
+                if (brief) A.set_done[set] = !bad;
+                if (!(brief && bad)) write_result(A.out + set, best, algo, bad);
+            }
         }
         team_sync();
     }

@@ -224,13 +224,15 @@ size_t direct_f32_bytes(int n);
 cudaError_t launch_direct_f32(const float *x, const float *y, int n, int h, int algo, lms_result *out, int *done,
                               void *mem, cudaStream_t st);
 // Many sets of at most nmax <= DIRECT_BATCH_MAX points, one CTA each: sets
-// (device) lists the set indices in the order they are handed out.
+// (device) lists the set indices in the order they are handed out.  A set of
+// at most small_max points that takes long is left to another kernel:
+// set_done[set] is 1 when its record is written, else 0.
 constexpr int DIRECT_BATCH_MAX = 4096;
 int direct_batch_teams(int nsets, int nmax, int sms);   // resident CTAs, 0 on failure
 size_t direct_batch_bytes(int nteams, int nmax);
 cudaError_t launch_direct_batch(const short *x, const short *y, const long long *off, const int *hvec, const int *sets,
-                                int nsets, int nmax, int nteams, int plain_max, int bnb_min, lms_result *out,
-                                void *mem, cudaStream_t st);
+                                int nsets, int nmax, int nteams, int plain_max, int bnb_min, int *set_done,
+                                int small_max, lms_result *out, void *mem, cudaStream_t st);
 
 // ---------------------------------------------------------------- argmin
 cudaError_t launch_argmin(const Cand *cands, int count, lms_result *out, int algorithm, const int *err,

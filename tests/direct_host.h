@@ -72,6 +72,7 @@ static inline float __ll2float_ru(long long v)
     return (long double)r < (long double)v ? nextafterf(r, INFINITY) : r;
 }
 static inline float __fmul_rn(float a, float b) { return a * b; }
+static inline float __fdividef(float a, float b) { return a / b; }
 static inline float __frcp_rn(float a) { return 1.0f / a; }
 static inline unsigned __float2uint_rz(float f) { return (unsigned)f; }
 static inline int __double2int_rn(double v) { return (int)nearbyint(v); }

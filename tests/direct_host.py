@@ -36,8 +36,11 @@ extern "C" void host_i16(const short *x, const short *y, int n, int h, int batch
 {
     DirectArgs a = {};
     a.x = x; a.y = y; a.n = n; a.h = h; a.out = out;
+    int done = -1;
+    if (batch == 2) { a.set_done = &done; a.small_max = n; }
     if (batch) host_fit<false>(a, 2048, 64, 32, 256.0f);
     else host_fit<false>(a, 4096, 256, 64, 256.0f);
+    host_count[0][7] = done;
     memcpy(count, host_count, sizeof host_count);
 }
 extern "C" int host_f32(const float *x, const float *y, int n, int h, lms_result *out, long long *count)
@@ -83,11 +86,13 @@ class Direct:
         done = f(p[0], p[1], x.size, h or x.size // 2 + 1, *extra, p[2], p[3])
         calls = dict(zip(MODES, count[0].tolist()))
         calls["phases"] = sum(calls[m] for m in MODES[:4])
+        calls["done"] = int(count[0, 7])
         calls.update({m + "_sum": v for m, v in zip(MODES, count[1].tolist())})
         return done, rec[0], calls
 
-    def i16(self, x, y, h=0, batch=False):
-        """The record and the counters of one fit, in the shape of small single fits or of a batch's sets."""
+    def i16(self, x, y, h=0, batch=0):
+        """The record and the counters of one fit: in the shape of small single fits (batch 0), of a batch's sets (1), of
+        its small sets, which may be left to the plain kernel (2; then calls["done"] is 0)."""
         x, y = (np.ascontiguousarray(v, dtype=np.int16) for v in (x, y))
         return self._run(self.lib.host_i16, x, y, h, int(batch))[1:]
 

@@ -23,7 +23,7 @@ def test_int16_equals_oracle(D, orc, kind):
         x, y = x.astype(np.int16), y.astype(np.int16)
         for h in sorted({1, 2, n // 8 + 1, n // 2 + 1, int(0.75 * n) + 1, n} & set(range(1, n + 1))):
             want = orc.lms_i16(x, y, h, "brute" if n <= 160 else "sweep")
-            for batch in (False, True):
+            for batch in (0, 1):
                 r, _ = D.i16(x, y, h, batch)
                 assert tuple(int(r[k]) for k in EXACT) == tuple(want.exact()), (kind, n, h, batch, r, want)
 
@@ -45,6 +45,24 @@ def test_shared_widths_are_not_scored_as_fractions(D):
     fractions, most of them no pair's slope)."""
     _, c = D.i16(*points("vertical", 8192, 8192), 6144)
     assert c["exact_sum"] <= 16384 and c["phases"] <= 256, c
+
+
+@pytest.mark.parametrize("kind", ["line", "sloped", "pure", "random", "full", "digital", "columns", "duplicates",
+                                  "vertical", "two_lines"])
+def test_small_sets_of_a_batch_end_early(D, orc, kind):
+    """Sets of 97 to 256 points finish, or are left to the plain kernel after a bounded number of phases; ordinary ones
+    finish."""
+    for n in (97, 128, 200, 256):
+        for seed in range(6):
+            x, y = (v.astype(np.int16) for v in points(kind, n, 100 * n + seed))
+            for h in (0, int(0.75 * n), n // 3 + 1):
+                r, c = D.i16(x, y, h, 2)
+                assert c["phases"] <= 22, (n, seed, h, c)
+                if c["done"]:
+                    want = orc.lms_i16(x, y, h, "brute" if n <= 128 else "sweep")
+                    assert tuple(int(r[k]) for k in EXACT) == tuple(want.exact())
+                else:
+                    assert kind in ("columns", "duplicates", "vertical", "two_lines", "pure"), (n, seed, h, c)
 
 
 # ---------------------------------------------------------------- float sets
