@@ -849,8 +849,10 @@ __device__ __forceinline__ bool candidates_above(float v, float limit, int *s_wa
         for (int d = 16; d >= 1; d >>= 1) v += __shfl_xor_sync(FULL, v, d);
         if ((threadIdx.x & 31) == 0) s_warp[threadIdx.x >> 5] = __float_as_int(v);
         __syncthreads();
-        v = 0.0f;
-        for (int w = 0; w < T / 32; ++w) v += __int_as_float(s_warp[w]);
+        const int lane = threadIdx.x & 31;
+        v = lane < T / 32 ? __int_as_float(s_warp[lane]) : 0.0f;
+#pragma unroll
+        for (int d = 16; d >= 1; d >>= 1) v += __shfl_xor_sync(FULL, v, d);
         __syncthreads();
     }
     return v > limit;
@@ -975,7 +977,9 @@ __device__ __forceinline__ int fraction_q(long long A, long long B, int xr, int 
 // Expected reduced fractions p / q of such a leaf: about 0.31 q^2 times its width.
 __device__ __forceinline__ float fractions(long long A, long long B, int xr, int yr)
 {
-    const float q = (float)fraction_q(A, B, xr, yr);
+    // (fraction_q in float: it is asked for every interval)
+    const float nearest = A > 0 ? (float)A : B < 0 ? -(float)B : 0.0f;
+    const float q = nearest > 0.0f ? fminf((float)xr, __fdividef(4294967296.0f * (float)(yr + 1), nearest) + 1.0f) : (float)xr;
     return 0.31f * q * q * (float)(B - A) * (1.0f / 4294967296.0f);
 }
 
@@ -984,6 +988,38 @@ __device__ __forceinline__ float leaf_slopes(const DNode &lf, float gain, int xr
 {
     const float f = fractions(lf.a, lf.b, xr, yr), e = fmaxf(lf.est * gain, 1.0f);
     return f < FRACTIONS ? fminf(f + 1.0f, 4.0f * e + LEAF_FRACTIONS) : e;
+}
+
+// How many of the count leaves together are expected to list at most limit
+// slopes (one at least), and how many slopes those are: every warp for itself,
+// a leaf a lane.
+template <int T, bool F>
+__device__ __forceinline__ int leaves_within(const DNode *leaf, int count, float limit, float gain, int xr, int yr,
+                                             float &slopes)
+{
+    constexpr int L = T >= 32 ? 32 : 1;
+    const int lane = threadIdx.x % L;
+    slopes = 0.0f;
+    for (int l0 = 0; l0 < count; l0 += L) {
+        const int l = l0 + lane;
+        float v = 0.0f;
+        if (l < count) v = F ? fmaxf(leaf[l].est * gain, 1.0f) : leaf_slopes(leaf[l], gain, xr, yr);
+        if constexpr (L == 32) {
+#pragma unroll
+            for (int d = 1; d < 32; d <<= 1) {
+                const float o = __shfl_up_sync(FULL, v, d);
+                if (lane >= d) v += o;
+            }
+        }
+        const unsigned beyond = __ballot_sync(FULL, l > 0 && l < count && slopes + v > limit);
+        if (beyond) {
+            const int first = __clz((int)(beyond & (0u - beyond))) ^ 31;
+            if (first > 0) slopes += __shfl_sync(FULL, v, (first - 1) % L);
+            return l0 + first;
+        }
+        slopes += __shfl_sync(FULL, v, L - 1);
+    }
+    return count;
 }
 
 // Shared bytes of list_pairs for NC cells and n points.
@@ -1002,17 +1038,16 @@ __host__ __device__ constexpr size_t pairs_bytes(int NC, int n)
 // g = -A q mod 2^32 is below (B - A) q: two 32-bit products a q, whatever the
 // number of points (n = 65536, 10 leaves: 4.6 ms by pairs).  Otherwise the
 // pairs are found by cells (see the head of the file); so are they when the
-// leaves listed together hold more fractions than the list and this one far
-// more than the pairs expected (most fractions are then no pair's slope, and
-// each would be tested and scored).  Cells that hold many points hold
+// leaf holds far more fractions than the pairs expected (most fractions are
+// then no pair's slope, and each would be tested and scored).  Cells that hold many points hold
 // quadratically many candidates with few distinct slopes.  Above the limit
 // nothing is searched: points that repeat another one are left out (dup, once
 // they are marked: 2048 points, 70% of them at one place, cost 35 ms of
 // candidates), and for points on one line the leaf is tried by fractions, or
 // false is returned and it is cut until it can be.
 template <int T>
-__device__ __noinline__ bool list_pairs(const int *pts, int n, const unsigned *dup, const DNode &lf, bool by_fractions,
-                                        const Box &bx, int NC, unsigned char *wk, int *s_warp, const TeamMem &m,
+__device__ __noinline__ bool list_pairs(const int *pts, int n, const unsigned *dup, const DNode &lf, const Box &bx, int NC,
+                                        unsigned char *wk, int *s_warp, const TeamMem &m,
                                         int *nlist, int *over, int HC,
                                         int part, int parts)
 {
@@ -1038,7 +1073,7 @@ __device__ __noinline__ bool list_pairs(const int *pts, int n, const unsigned *d
         }
     };
     const float fr = fractions(A, B, xr, yr);
-    if (fr < FRACTIONS && (by_fractions || fr <= 4.0f * fmaxf(lf.est, 1.0f) + LEAF_FRACTIONS)) {
+    if (fr < FRACTIONS && fr <= 4.0f * fmaxf(lf.est, 1.0f) + LEAF_FRACTIONS) {
         by_q();
         return true;
     }
@@ -1253,6 +1288,21 @@ __device__ __noinline__ void list_pairs_f32(const int2 *pts, int n, long long A,
     }
     __syncthreads();
     if (!want) table_append<T>(tab, m, nlist, over, HC, s_warp);
+}
+
+// The best of the CTA's candidates (buf: one a warp).
+template <int T>
+__device__ __forceinline__ Cand cta_best(Cand c, Cand *buf)
+{
+    if constexpr (T >= 32) {
+        c = warp_best(c);
+        if ((threadIdx.x & 31) == 0) buf[threadIdx.x >> 5] = c;
+        __syncthreads();
+        c = (threadIdx.x & 31) < T / 32 ? buf[threadIdx.x & 31] : cand_empty();
+        c = warp_best(c);
+        __syncthreads();
+    }
+    return c;
 }
 
 // The smallest width of the CTA's threads and the first window that has it.
@@ -2204,23 +2254,14 @@ __global__ void __launch_bounds__(T) k_direct(const DirectArgs A)
                 int NC = T;
                 while (NC < n && NC < CELLS_MAX) NC <<= 1;
                 const int parts = max(1, (int)C / lfn);
-                [[maybe_unused]] bool by_fractions = true;
-                if constexpr (!F) {
-                    float held = 0.0f;
-                    for (int l = lf0; l < lf0 + lfn; ++l) {
-                        const float f = fractions(S.leaf[l].a, S.leaf[l].b, xr, yr);
-                        if (f < FRACTIONS) held += f;
-                    }
-                    by_fractions = held <= 0.75f * (float)sh.HC;
-                }
                 for (int l = rank; l < lfn * parts; l += C) {
                     const DNode &lf = S.leaf[lf0 + l / parts];
                     if constexpr (F)
                         list_pairs_f32<T>(pts, n, lf.a, lf.b, bx, fs, NC, wk, S.warp_a, m, &st->nlist[lpar],
                                           &st->over[lpar], sh.HC, l % parts, parts);
                     else {
-                        const bool listed = list_pairs<T>(pts, n, marked ? m.dup : nullptr, lf, by_fractions, bx, NC, wk,
-                                                          S.warp_a, m, &st->nlist[lpar], &st->over[lpar], sh.HC,
+                        const bool listed = list_pairs<T>(pts, n, marked ? m.dup : nullptr, lf, bx, NC, wk, S.warp_a,
+                                                          m, &st->nlist[lpar], &st->over[lpar], sh.HC,
                                                           l % parts, parts);
                         if (threadIdx.x == 0 && l % parts == 0) {
                             m.ans[l / parts].dense = !listed;   // (no test runs here; LC <= 2 PM answers)
@@ -2233,9 +2274,8 @@ __global__ void __launch_bounds__(T) k_direct(const DirectArgs A)
                 const int nn = __ldcg(&st->nlist[lpar]);
                 // slopes to expect for each pair expected: few where many pairs share a slope
                 {
-                    float held = 0.0f;
-                    for (int l = lf0; l < lf0 + lfn; ++l)
-                        held += F ? S.leaf[l].est * gain : leaf_slopes(S.leaf[l], gain, xr, yr);
+                    float held;
+                    leaves_within<T, F>(S.leaf + lf0, lfn, 1e30f, gain, xr, yr, held);
                     if (F && (over == 2 || (over && (++cuts_more > F_CUTS || (lfn == 1 && S.leaf[lf0].b - S.leaf[lf0].a == 1)))))
                         err = 1;   // more slopes or candidates than the sweep is worth
                     if (over == 1 && lfn == 1) gain = fminf(64.0f, 4.0f * gain);
@@ -2434,11 +2474,14 @@ __global__ void __launch_bounds__(T) k_direct(const DirectArgs A)
                 // the best of them that is a pair's slope (fractions need not be)
                 for (int tries = 0; tries < nx; ++tries) {
                     Cand c = cand_empty();
-                    int at = -1;
-                    for (int k = 0; k < nx; ++k) {
-                        const Cand o = ld_cand(&m.xres[k]);
-                        if (S.xl[k] >= 0 && cand_better(o, c)) { c = o; at = k; }
+                    for (int k = threadIdx.x; k < nx; k += T) {
+                        Cand o = ld_cand(&m.xres[k]);
+                        o.i = k;
+                        if (S.xl[k] >= 0 && cand_better(o, c)) c = o;
                     }
+                    c = cta_best<T>(c, reinterpret_cast<Cand *>(S.red));
+                    const int at = c.i;
+                    c.i = c.j = 0x7fffffff;   // (an equal slope is not better)
                     if (!cand_better(c, best)) break;
                     line_pair<T>(pts, n, c.dy, c.dx, reinterpret_cast<unsigned *>(wk), slots, rounds, (int)rank, (int)C,
                                  &st->pair[ppar], &st->bad);
@@ -2493,16 +2536,9 @@ __global__ void __launch_bounds__(T) k_direct(const DirectArgs A)
                     P = 0;
                 }
                 // as many of the leaves as the list is expected to hold
-                lfn = min(nleaf - lf0, lcap);
-                {
-                    float held = 0.0f;
-                    int l = 0;
-                    for (; l < lfn; ++l) {
-                        held += F ? fmaxf(S.leaf[lf0 + l].est * gain, 1.0f) : leaf_slopes(S.leaf[lf0 + l], gain, xr, yr);
-                        if (l > 0 && held > LIST_HOPE * (float)sh.HC) break;
-                    }
-                    lfn = max(1, l);
-                }
+                float held;
+                lfn = leaves_within<T, F>(S.leaf + lf0, min(nleaf - lf0, lcap), LIST_HOPE * (float)sh.HC, gain, xr, yr,
+                                          held);
                 flush = true;
             } else if (was_tree && P > 0) {
                 mode = M_TREE;
