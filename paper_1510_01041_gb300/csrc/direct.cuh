@@ -1022,6 +1022,18 @@ __device__ __forceinline__ int leaves_within(const DNode *leaf, int count, float
     return count;
 }
 
+// First position of share `part` of the held points in ord, which lie cell by
+// cell (end[q]: where cell q ends): whole cells.  CTAs that share a leaf sort
+// the points into cells each for itself, and the order inside a cell differs
+// between them, so a cell cut between two of them would lose pairs.
+template <class CELL>
+__device__ __forceinline__ int share_start(int part, int parts, int held, const unsigned *end, const unsigned short *ord,
+                                           CELL cell_of)
+{
+    const int p = (int)((long long)held * part / parts);
+    return p == 0 ? 0 : (int)end[cell_of(ord[p - 1])];
+}
+
 // Shared bytes of list_pairs for NC cells and n points.
 __host__ __device__ constexpr size_t pairs_bytes(int NC, int n)
 {
@@ -1127,10 +1139,13 @@ __device__ __noinline__ bool list_pairs(const int *pts, int n, const unsigned *d
         // then the next cell) end to end and tests 32 of them at once.
         constexpr int L = T >= 32 ? 32 : 1;
         const int lane = threadIdx.x % L;
-        for (int e0 = part * T + threadIdx.x - lane; e0 < held; e0 += T * parts) {
+        auto cell_of = [&](int k) { return cell(pts[k]); };
+        const int first = share_start(part, parts, held, cnt, ord, cell_of);
+        const int last = share_start(part + 1, parts, held, cnt, ord, cell_of);
+        for (int e0 = first + threadIdx.x - lane; e0 < last; e0 += T) {
             const int e = e0 + lane;
             int pa = 0, n1 = 0, nn = 0, beg2 = 0;
-            if (e < held) {
+            if (e < last) {
                 pa = pts[ord[e]];
                 const int q = cell(pa), q2 = (q + 1) & (NC - 1);
                 beg2 = q2 ? (int)cnt[q2 - 1] : 0;
@@ -1259,7 +1274,10 @@ __device__ __noinline__ void list_pairs_f32(const int2 *pts, int n, long long A,
     __syncthreads();
     const long long err = (1LL << F_YS) + ka + 4;
     constexpr int L = T >= 32 ? 8 : 1;
-    for (int e = (part * T + (int)threadIdx.x) / L; e < n; e += T * parts / L) {
+    auto cell_of = [&](int k) { return cell(pts[k]); };
+    const int first = share_start(part, parts, n, cnt, ord, cell_of);
+    const int last = share_start(part + 1, parts, n, cnt, ord, cell_of);
+    for (int e = first + (int)threadIdx.x / L; e < last; e += T / L) {
         const int a = ord[e];
         const int2 pa = pts[a];
         const int q = cell(pa), q2 = (q + 1) & (NC - 1);

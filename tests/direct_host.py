@@ -52,6 +52,52 @@ extern "C" int host_f32(const float *x, const float *y, int n, int h, lms_result
     memcpy(count, host_count, sizeof host_count);
     return done;
 }
+// The distinct slopes of a leaf listed by `parts` CTAs, each with the points in another order (as their cells may have
+// them): slope keys, or order words for float points.  Returns how many were listed, -1 if they did not fit.
+static TeamMem list_memory(std::vector<long long> &keys, std::vector<unsigned> &den)
+{
+    TeamMem m = {};
+    keys.resize(1 << 20);
+    den.resize(1 << 20);
+    m.lkey = keys.data();
+    m.lden = den.data();
+    return m;
+}
+extern "C" int host_list_i16(const int *pts, int n, long long A, long long B, int xr, int yr, int parts, long long *out)
+{
+    std::vector<long long> keys;
+    std::vector<unsigned> den;
+    TeamMem m = list_memory(keys, den);
+    Box bx = {0, 0, -xr, xr, -yr, yr, 0};
+    DNode lf = {A, B, 1, 0, 0.0f, 0};
+    int nlist = 0, over = 0, warp[32];
+    for (int part = 0; part < parts; ++part)
+        if (!list_pairs<1>(pts + (long long)part * n, n, nullptr, lf, bx, 1024, dsm, warp, m, &nlist, &over, 1 << 20,
+                           part, parts))
+            return -1;
+    memcpy(out, keys.data(), sizeof(long long) * nlist);
+    return over ? -1 : nlist;
+}
+extern "C" int host_list_f32(const float *xy, int n, long long A, long long B, int parts, long long *out)
+{
+    std::vector<long long> keys;
+    std::vector<unsigned> den;
+    TeamMem m = list_memory(keys, den);
+    int nlist = 0, over = 0, warp[32];
+    for (int part = 0; part < parts; ++part) {
+        const float *x = xy + 2LL * part * n, *y = x + n;
+        FloatSet f{};
+        Box bx;
+        long long red[8];
+        if (!float_box<1>(x, y, n, f, bx, red)) return -1;
+        std::vector<int2> pts(n);
+        for (int k = 0; k < n; ++k)
+            pts[k] = make_int2(__double2int_rn((x[k] - f.xc) * f.sx), __double2int_rn((y[k] - f.yc) * f.sy));
+        list_pairs_f32<1>(pts.data(), n, A, B, bx, f, 1024, dsm, warp, m, &nlist, &over, 1 << 20, part, parts);
+    }
+    memcpy(out, keys.data(), sizeof(long long) * nlist);
+    return over ? -1 : nlist;
+}
 """
 
 
@@ -100,6 +146,30 @@ class Direct:
         """Whether the attempt finished, its record and its counters."""
         x, y = (np.ascontiguousarray(v, dtype=np.float32) for v in (x, y))
         return self._run(self.lib.host_f32, x, y, h)
+
+    def listed_i16(self, x, y, lo, hi, parts, seed=0):
+        """Slope keys of a leaf [lo, hi) listed by `parts` CTAs with the points in another order each."""
+        rng = np.random.default_rng(seed)
+        order = [rng.permutation(x.size) for _ in range(parts)]
+        pts = np.concatenate([(y[o].astype(np.int32) << 16) | (x[o].astype(np.int32) & 0xffff) for o in order])
+        pts = np.ascontiguousarray(pts, np.int32)
+        out = np.zeros(1 << 20, np.int64)
+        n = self.lib.host_list_i16(ctypes.c_void_p(pts.ctypes.data), x.size, ctypes.c_int64(lo), ctypes.c_int64(hi),
+                                   int(np.abs(x).max()), int(np.abs(y).max()), parts, ctypes.c_void_p(out.ctypes.data))
+        assert n >= 0
+        return set(out[:n].tolist())
+
+    def listed_f32(self, x, y, lo, hi, parts, seed=0):
+        """The same for float points and scaled slope keys: the slopes, as doubles."""
+        rng = np.random.default_rng(seed)
+        order = [rng.permutation(x.size) for _ in range(parts)]
+        xy = np.concatenate([np.concatenate([np.float32(x[o]), np.float32(y[o])]) for o in order])
+        out = np.zeros(1 << 20, np.int64)
+        n = self.lib.host_list_f32(ctypes.c_void_p(xy.ctypes.data), x.size, ctypes.c_int64(lo), ctypes.c_int64(hi), parts,
+                                   ctypes.c_void_p(out.ctypes.data))
+        assert n >= 0
+        w = out[:n]
+        return set(np.where(w < 0, w ^ 0x7fffffffffffffff, w).view(np.float64).tolist())
 
 
 def load(folder):

@@ -28,6 +28,33 @@ def test_int16_equals_oracle(D, orc, kind):
                 assert tuple(int(r[k]) for k in EXACT) == tuple(want.exact()), (kind, n, h, batch, r, want)
 
 
+@pytest.mark.parametrize("parts", [1, 2, 5, 8, 16])
+def test_shared_leaf_loses_no_slope(D, parts):
+    """CTAs that share a leaf list all its slopes between them, whatever the order of the points inside the cells, which
+    differs between CTAs."""
+    rng = np.random.default_rng(parts)
+    for n in (40, 200, 700):
+        x, y = rng.integers(-30000, 30001, n), rng.integers(-30000, 30001, n)
+        i, j = np.triu_indices(n, 1)
+        ok = x[i] != x[j]
+        i, j = i[ok], j[ok]
+        dx, dy = x[j] - x[i], y[j] - y[i]
+        keys = ((np.where(dx < 0, -dy, dy).astype(object) << 32) // np.abs(dx)).astype(np.int64)
+        lo, hi = np.sort(keys)[[keys.size // 2, keys.size // 2 + 300]].tolist()
+        want = set(keys[(keys >= lo) & (keys < hi)].tolist())
+        for seed in range(4):
+            assert D.listed_i16(x, y, lo, hi, parts, seed) == want, (n, seed)
+        # float points: the frame scales both axes by powers of two
+        xf, yf = np.float32(x + rng.random(n)), np.float32(y + rng.random(n))
+        s = np.subtract(yf[j], yf[i], dtype=np.float64) / np.subtract(xf[j], xf[i], dtype=np.float64)
+        ex, ey = (np.frexp(np.float64(v.max()) - np.float64(v.min()))[1] for v in (xf, yf))
+        k = s * 2.0 ** (int(ex) - int(ey)) * 2.0 ** 29
+        lo, hi = np.floor(np.sort(k)[[k.size // 2, k.size // 2 + 300]]).astype(np.int64).tolist()
+        wantf = set(s[(k >= lo) & (k < hi)].tolist())
+        for seed in range(4):
+            assert D.listed_f32(xf, yf, lo, hi, parts, seed) == wantf, (n, seed)
+
+
 # The counters of ordinary sets at these sizes: at most 16 phases, 32 candidates a point and leaf, 10 slopes scored.
 @pytest.mark.parametrize("kind,n,h", [("duplicates", 2048, 0), ("duplicates", 513, 0), ("two_lines", 4096, 4096),
                                       ("pure", 2048, 267), ("rows", 2048, 0), ("collinear", 4096, 0)])
