@@ -77,11 +77,12 @@ class Host:
 
 
 def load(folder):
-    """Links the built objects to the stand-in runtime; a fresh library (its own state) in `folder`."""
+    """Links the built objects to the stand-in runtime (bound to itself: another runtime may be loaded); a fresh library
+    with its own state in `folder`."""
     build.build()
     cuda = os.path.dirname(os.path.dirname(os.path.realpath(build.nvcc())))
     path = os.path.join(str(folder), "liblms_host.so")
-    subprocess.run(["g++", "-std=c++17", "-O1", "-shared", "-fPIC", "-I", os.path.join(cuda, "include"), "-o", path,
+    subprocess.run(["g++", "-std=c++17", "-O1", "-shared", "-fPIC", "-Wl,-Bsymbolic", "-I", os.path.join(cuda, "include"), "-o", path,
                     os.path.join(HERE, "fake_cudart.cpp"), *sorted(glob.glob(os.path.join(build.OUT, "*.o")))],
                    check=True)
     return Host(path)
