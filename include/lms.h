@@ -71,8 +71,11 @@ enum lms_dtype {
 };
 
 enum lms_algo {
-    LMS_ALGO_AUTO = 0,        /* library choice; reports PLAIN (int16 up to 512 points) or SWEEP, whose record it
-                                 equals, also where a branch-and-bound drops slopes that cannot win */
+    LMS_ALGO_AUTO = 0,        /* library choice; reports PLAIN (int16 up to 512 points) or SWEEP also where a
+                                 branch-and-bound drops slopes that cannot win.  For int16 the record equals
+                                 theirs bit for bit; for float the line is a best one in double arithmetic,
+                                 whose width equals the sweep's up to the rounding of the projections (2^-50 of
+                                 the largest |y| + 2 |theta1 x|) */
     LMS_ALGO_PLAIN = 1,       /* sort the projections at every pairwise slope (n <= 1024) */
     LMS_ALGO_SWEEP = 2,       /* exact kinetic sweep over slope-sorted events */
     LMS_ALGO_BNB = 3,         /* seeded branch-and-bound over slope intervals + sweep of survivors */
@@ -100,7 +103,9 @@ typedef struct {
     double med_sq;            /* (w/2)^2: the h-th smallest squared residual */
     int32_t i, j;             /* smallest pair (i < j) with slope theta1; -1 if none */
     int32_t status;           /* enum lms_status for this fit */
-    int32_t algorithm;        /* enum lms_algo that produced it */
+    int32_t algorithm;        /* enum lms_algo: the method the call asked for, or PLAIN, SWEEP or BNB by the
+                                 size and options (the one-kernel branch-and-bound reports the method it
+                                 stands in for) */
 } lms_result;
 
 /*
@@ -220,13 +225,18 @@ LMS_API int lms_fit_learned_host(lms_setnet *net, const void *x, const void *y, 
 /*
  * Batched fits of many point sets of uneven size (not in the paper: its
  * Hough application runs one LMS per accumulator peak; this runs them all).
- * lms_batch_plan_create sizes everything from the host offsets once: sets
- * with at most plain_max_n points (0 = 256, at most 256) go to one
- * persistent plain kernel over (set, run of slopes) work items in three
- * size classes (up to 64 points; above, to one CTA of the one-kernel
- * branch-and-bound, with the same record); larger sets (up to 32768 points) each get the exact sweep
- * of every slope or, from 512 points on, the exact branch-and-bound, spread
- * over `streams` internal streams (0 = 8).  It allocates the plan's
+ * lms_batch_plan_create sizes everything from the host offsets once.  With
+ * plain_max_n 0 (the library's choice) sets below 97 points, and those of up
+ * to 256 with an order statistic below n / 3, go to one persistent plain
+ * kernel over (set, run of slopes) work items in three size classes; sets of
+ * 97 to 4096 points each get one CTA of the one-kernel branch-and-bound (one
+ * launch for all; the plain kernel finishes those of up to 256 points that
+ * would take it long); the rest, up to 32768 points, the exact
+ * branch-and-bound of many kernels (from 512 points on) or the sweep of every
+ * slope, spread over `streams` internal streams (0 = 8).  With plain_max_n > 0
+ * (at most 256) sets of up to that size go to the plain kernel.  Every path
+ * gives the same record; its `algorithm` is PLAIN up to plain_max_n points
+ * (0: 256), BNB from bnb_min_n on, else SWEEP.  The call allocates the plan's
  * device memory and waits for the device.
  *   offsets_host  B + 1 offsets of the sets in the x/y arrays (host).
  *   h_host        per-set order statistic (NULL: floor(n/2) + 1 each).
@@ -239,11 +249,11 @@ LMS_API int lms_fit_learned_host(lms_setnet *net, const void *x, const void *y, 
 typedef struct lms_batch_plan lms_batch_plan;
 LMS_API int lms_batch_plan_create(const int64_t *offsets_host, int64_t B, const int32_t *h_host,
                                   int32_t plain_max_n, int32_t streams, lms_batch_plan **plan);
-/* The same with the size from which a set is fitted by the exact
- * branch-and-bound (lms_fit_bnb's method, asynchronous, without statistics)
- * instead of the sweep of every slope: bnb_min_n 0 = 512 points (the value
- * lms_batch_plan_create uses), > 0 = that size (at least 257), < 0 = never.
- * The branch-and-bound's result equals the sweep's bit for bit. */
+/* The same with the size from which a set is fitted by an exact
+ * branch-and-bound (lms_fit_bnb's method, asynchronous, without statistics):
+ * bnb_min_n 0 = the library's choice (what lms_batch_plan_create does),
+ * > 0 = from that size on (at least 257), the sweep of every slope below,
+ * < 0 = never.  The branch-and-bound's result equals the sweep's bit for bit. */
 LMS_API int lms_batch_plan_create_ex(const int64_t *offsets_host, int64_t B, const int32_t *h_host,
                                      int32_t plain_max_n, int32_t streams, int32_t bnb_min_n,
                                      lms_batch_plan **plan);

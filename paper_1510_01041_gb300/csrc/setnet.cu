@@ -557,8 +557,10 @@ int lms_fit_learned(lms_setnet *net, const void *x, const void *y, int64_t n, in
         }
     }
     // the forward pass runs on the net's side stream, forked from and joined
-    // back to `stream`: the branch-and-bound samples and sorts pair slopes
-    // meanwhile and waits for the prediction only where it picks its seeds
+    // back to `stream`: with statistics, seed modes or a small order statistic
+    // the branch-and-bound of many kernels samples and sorts pair slopes
+    // meanwhile and waits for the prediction only where it picks its seeds; the
+    // one kernel waits for it before its launch
     if (cudaEventRecord(net->ev_fork, st) != cudaSuccess || cudaStreamWaitEvent(net->side, net->ev_fork, 0) != cudaSuccess)
         return LMS_ERR_CUDA;
     {
