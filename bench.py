@@ -10,8 +10,8 @@ oracle):
 
 * ``learned``       (headline ``value``) lms_fit_learned: the set network
                     predicts the slope, branch-and-bound takes its upper bound
-                    there, drops slope intervals whose lower bound exceeds it,
-                    and sweeps the rest exactly;
+                    there, drops slope intervals that cannot be narrower and
+                    scores the slopes left exactly, all in one kernel;
 * ``quantile_bnb``  lms_fit_bnb without a network: the same branch-and-bound
                     seeded at quantiles of sampled pair slopes;
 * ``plain``         lms_fit with the kinetic sweep over every candidate slope.
@@ -468,8 +468,8 @@ def _timed(fit, steps, warmup, flush, stream, barrier):
 
 
 def batched_short(steps: int, warmup: int):
-    """The batch workload (4096 uneven sets) with a fixed plan (plain kernel up
-    to 128 points, 48 streams, branch-and-bound from 512 points), captured
+    """The batch workload (4096 uneven sets) with the library's own choice of
+    paths (the plain kernel below 97 points, one kernel from there), captured
     into one CUDA graph; each step replays it on a fresh batch already in HBM
     (y coordinates of another seed), timed with CUDA events."""
     import numpy as np
@@ -482,7 +482,7 @@ def batched_short(steps: int, warmup: int):
     y1 = (y0.astype(np.int64) + datagen.Stream(5001).integers(-2, 3, y0.size)).clip(-32768, 32767).astype(np.int16)
     xt, yt, ot = (torch.from_numpy(a).to(dev) for a in (x0, y0, off))
     ys = [torch.from_numpy(y0).to(dev), torch.from_numpy(y1).to(dev)]
-    plan = lms.BatchPlan(off, plain_max_n=128, streams=48, bnb_min_n=512)
+    plan = lms.BatchPlan(off)
     out = torch.empty((4096, lms.RESULT_DTYPE.itemsize), dtype=torch.uint8, device=dev)
     plan.fit(xt, yt, ot, out=out)
     torch.cuda.synchronize()
@@ -511,7 +511,7 @@ def batched_short(steps: int, warmup: int):
     return {"value": v, "unit": UNIT, "ms_per_step": ms / steps, "candidate_slopes_per_sec": v / 4096 * slopes,
             "steps": steps, "warmup": warmup,
             "workload": "4096 sets, n log-uniform [64,4096], outliers U(0,0.45), angle U(-1.5,1.5)",
-            "plan": "plain kernel <= 128 points, 48 streams, branch-and-bound >= 512 points, one CUDA graph"}
+            "plan": "library defaults: plain kernel below 97 points, one-kernel branch-and-bound above, one CUDA graph"}
 
 
 def hough_short(steps: int, warmup: int):
@@ -571,7 +571,7 @@ def _roof(stage, stages, units_per_fit, ops_per_unit, fits, peak_tops, mhz_basis
 # the kernel, and its DRAM traffic per launch (dram__bytes_read.sum +
 # dram__bytes_write.sum) from the ncu captures summarised under profiles/;
 # a kernel changed after its capture has no entry.
-KERNEL_OF_STAGE = {"sweep": "k_sweep", "node_bounds": "k_node_lb"}
+KERNEL_OF_STAGE = {"sweep": "k_sweep", "node_bounds": "k_node_lb", "direct": "k_direct"}
 DRAM_BYTES = {"k_node_lb": 152_320, "k_sweep": 386_048, "k_sweep_plain": 194_637_824}
 
 
@@ -714,7 +714,8 @@ def main():
         _timed(arms[k], args.steps, args.warmup, flush, stream, barrier)
         stages[k] = lms.profile_read()
     lms.profile_enable(False)
-    # statistics of the branch-and-bound fits (untimed)
+    # statistics of the staged branch-and-bound on the same sets (untimed: the
+    # timed fits ask for none and run as one kernel)
     for s in range(args.warmup, args.warmup + args.steps):
         stats["learned"].append(net.fit(xs[s], ys[s], 0, out=outs["learned"][s])[1])
         stats["quantile"].append(lms.fit_bnb(xs[s], ys[s], 0, None, out=outs["quantile"][s],
@@ -755,6 +756,10 @@ def main():
     mean = lambda arm, k: float(np.mean([st[k] for st in stats[arm]])) if stats[arm] else 0.0
     roofs = {}
     for arm, st in (("learned", stages["learned"]),):
+        # the one kernel of the timed fits: the operations a fit cannot do without
+        # (two a point and one sorting step); what it spends is its chain of phases
+        roofs["direct"] = _roof("direct", st, 2.0 * N_POINTS + N_POINTS * math.log2(N_POINTS), 1, args.steps, peak,
+                                basis, None)
         roofs["sweep"] = _roof("sweep", st, mean(arm, "events_swept"), SWEEP_INT_OPS_PER_EVENT, args.steps, peak,
                                basis, DRAM_BYTES.get("k_sweep"))
         roofs["node_bounds"] = _roof("node_bounds", st, mean(arm, "nodes_evaluated"), node_bound_ops(N_POINTS),
@@ -798,10 +803,12 @@ def main():
                                                            "(the method without the network)"}),
         "plain": arm_line("plain", {"algorithm": "kinetic sweep, every slope"}),
         "events_total_mean": mean("learned", "events_total"),
+        "statistics_from": "untimed fits by the staged branch-and-bound on the same sets; the timed learned and "
+                           "quantile fits are one kernel, which keeps no such counts",
         "line_40pct": {"workload": "line_with_outliers: slope 0.7, 40% outliers, n=8192",
                        "learned": arm_line("learned2"), "plain": arm_line("plain2")},
         "config": {"workload": WORKLOAD, "n": N_POINTS, "h": N_POINTS // 2 + 1,
-                   "algorithm": "learned-seeded branch-and-bound + sweep of surviving slopes",
+                   "algorithm": "learned-seeded branch-and-bound, one kernel a fit after the network",
                    "l2": "flushed before every step (256 MB write, outside the timed events)",
                    "launch": "learned and quantile-seeded fits: one CUDA graph per step, captured after "
                              "the warm-up and replayed; plain sweep and the 40% line workload: direct calls",

@@ -1,9 +1,11 @@
-"""Autotuner for batched fits: picks the size threshold between the plain
-kernel classes and the sweep, the number of sweep streams and the size from
-which sets take the branch-and-bound instead of the sweep, by timing
-CUDA-graph replays of a batch plan on the caller's own sets.  Results are
-cached per (device name, size mix) in autotune_cache.json next to this
-file, or in the file $LMS_AUTOTUNE_CACHE names.
+"""Autotuner for batched fits: the library's own choice of paths against given
+options (the size threshold of the plain kernel classes, the number of sweep
+streams, the size from which sets take a branch-and-bound instead of the
+sweep), by timing CUDA-graph replays of a batch plan on the caller's own sets.
+Only options that change what runs are tried: streams and the staged
+branch-and-bound serve sets above 4096 points.  Results are cached per (device
+name, size mix) in autotune_cache.json next to this file, or in the file
+$LMS_AUTOTUNE_CACHE names.
 
     from paper_1510_01041_gb300 import autotune
     plan, cfg = autotune.tuned_plan(offsets, x, y, offsets_dev)
@@ -23,9 +25,10 @@ from . import lms
 # cache that cannot be written is reported by a warning and tuning still works.
 CACHE = os.environ.get("LMS_AUTOTUNE_CACHE") or os.path.join(os.path.dirname(os.path.abspath(__file__)),
                                                              "autotune_cache.json")
-PLAIN_MAX = (64, 128, 256)
+PLAIN_MAX = (0, 64, 128, 256)         # 0: the library's choice
 STREAMS = (8, 16, 32, 48)
-BNB_MIN = (384, 512, 768, 1536, -1)   # -1: every large set takes the sweep of every slope
+BNB_MIN = (512, 1536, -1)             # -1: every large set takes the sweep of every slope
+ONE_KERNEL_MAX = 4096                 # points of the largest set fitted by one kernel
 
 
 def _key(offsets, device_name):
@@ -37,7 +40,7 @@ def _key(offsets, device_name):
     hist = np.histogram(np.log2(np.maximum(sizes, 2)), bins=128, range=(1, 17))[0]
     pairs = int(np.sum(sizes * (sizes - 1) // 2))
     h = hashlib.sha1(hist.tobytes() + device_name.encode()).hexdigest()[:16]
-    return f"v2:{device_name}:{sizes.size}:{int(sizes.sum())}:{pairs}:{h}"
+    return f"v3:{device_name}:{sizes.size}:{int(sizes.sum())}:{pairs}:{h}"
 
 
 def _time_plan(plan, x, y, od, reps=2):
@@ -61,9 +64,10 @@ def _time_plan(plan, x, y, od, reps=2):
 
 def tune(offsets, x, y, offsets_dev, candidates=None):
     """Time candidate plans (plain_max_n, streams, bnb_min_n); returns the
-    best config.  Coordinate search: the plain threshold and stream count at
-    the default branch-and-bound size, then the branch-and-bound size at the
-    best of those (or every given candidate)."""
+    best config.  Coordinate search: the plain threshold and, with sets above
+    4096 points, the stream count at the default branch-and-bound size, then
+    the branch-and-bound size at the best of those (or every given
+    candidate)."""
     import torch
     results = []
 
@@ -78,11 +82,12 @@ def tune(offsets, x, y, offsets_dev, candidates=None):
         for c in candidates:
             run(*c)
     else:
+        large = int(np.max(np.diff(np.asarray(offsets, dtype=np.int64)))) > ONE_KERNEL_MAX
         for pm in PLAIN_MAX:
-            for ns in STREAMS:
+            for ns in STREAMS if large else STREAMS[:1]:
                 run(pm, ns, 0)
         b = min(results, key=lambda r: r["seconds"])
-        for bm in BNB_MIN:
+        for bm in BNB_MIN if large else ():
             run(b["plain_max_n"], b["streams"], bm)
     best = min(results, key=lambda r: r["seconds"])
     return best, results
