@@ -1823,6 +1823,11 @@ struct DShared {
     Box bx;
     int nsmp, set;
     long long t0, t1;
+    // what listing has learned; kept here, not in registers, since every call of the
+    // loop below saves what is live (read before a barrier, written by thread 0 after it)
+    float gain;                  // slopes to expect for each pair expected
+    int lcap, regrown, cuts;     // leaves listed at a time; times that leaves or lists were cut
+    int marked;                  // duplicates are marked
 };
 
 // Children of a tree node: cut keys into c[1 .. count - 1] (c[0] = a, c[count] = b).
@@ -1967,8 +1972,8 @@ __global__ void __launch_bounds__(T) k_direct(const DirectArgs A)
             st->nlist[0] = st->nlist[1] = st->over[0] = st->over[1] = 0;
         }
         team_sync();
-        [[maybe_unused]] const bool brief = !F && A.set_done && n <= A.small_max;
-        const int phases = F ? F_PHASES : brief ? SMALL_PHASES : PHASES_MAX;
+        auto brief = [&]() { return !F && A.set_done && n <= A.small_max; };
+        auto phases = [&]() { return F ? F_PHASES : brief() ? SMALL_PHASES : PHASES_MAX; };
         const int algo = n <= A.plain_max ? LMS_ALGO_PLAIN : n >= A.bnb_min ? LMS_ALGO_BNB : A.algo;
         if constexpr (!F) {
         if (S.bx.xlo == S.bx.xhi) {
@@ -1978,7 +1983,7 @@ __global__ void __launch_bounds__(T) k_direct(const DirectArgs A)
                 c.i = c.j = -1;
                 if (threadIdx.x == 0) {
                     write_result(A.out + set, c, algo, 0);
-                    if (brief) A.set_done[set] = 1;
+                    if (brief()) A.set_done[set] = 1;
                 }
             }
             team_sync();
@@ -2112,15 +2117,24 @@ __global__ void __launch_bounds__(T) k_direct(const DirectArgs A)
             S.work[0][q] = nd;
         }
         // hash tables of line_pair and mark_duplicates
-        int slots = 1024, rounds = 1;
-        while (slots * 8 <= wk_bytes && slots < 2 * n) slots <<= 1;
-        while (rounds < (int)C || (long long)rounds * slots < 2LL * n) rounds <<= 1;
+        auto table_slots = [&]() {
+            int slots = 1024;
+            while (slots * 8 <= wk_bytes && slots < 2 * n) slots <<= 1;
+            return slots;
+        };
+        auto table_rounds = [&](int slots) {
+            int rounds = 1;
+            while (rounds < (int)C || (long long)rounds * slots < 2LL * n) rounds <<= 1;
+            return rounds;
+        };
+        if (threadIdx.x == 0) {
+            S.gain = 1.0f;
+            S.lcap = LC;
+            S.regrown = S.cuts = S.marked = 0;
+        }
         // the plan: the same values in every thread of the team
         int mode = M_TREE, P = Q + 1, cur = 0, par = 0, lpar = 0, ppar = 0;
-        int top = 0, etop = 0, nleaf = 0, lf0 = 0, lfn = 0, nx = 0, err = 0, regrown = 0, scored = 0, lcap = LC;
-        float gain = 1.0f;
-        [[maybe_unused]] int cuts_more = 0;
-        [[maybe_unused]] bool marked = false;   // duplicates are marked
+        int top = 0, etop = 0, nleaf = 0, lf0 = 0, lfn = 0, nx = 0, err = 0, scored = 0;
         bool flush = false;
         long long ux = D_MAX, uxl = D_MAX, bkey = D_MAX;
         Cand best = cand_empty();
@@ -2205,7 +2219,7 @@ __global__ void __launch_bounds__(T) k_direct(const DirectArgs A)
                     if (nd.b - nd.a == 1) return true;
                     if (nd.force > 0) return false;
                     const float f = F ? 0.0f : fractions(nd.a, nd.b, xr, yr);
-                    return nd.est * gain <= sh.leaf || (!F && f <= LEAF_FRACTIONS);
+                    return nd.est * S.gain <= sh.leaf || (!F && f <= LEAF_FRACTIONS);
                 };
                 const int pers = (ns + T - 1) / T;
                 const int i0 = min(ns, (int)threadIdx.x * pers), i1 = min(ns, i0 + pers);
@@ -2277,6 +2291,10 @@ __global__ void __launch_bounds__(T) k_direct(const DirectArgs A)
                 int NC = T;
                 while (NC < n && NC < CELLS_MAX) NC <<= 1;
                 const int parts = max(1, (int)C / lfn);
+                // (read here; thread 0 writes them behind the barrier)
+                float gain = S.gain;
+                int lcap = S.lcap, regrown = S.regrown, cuts_made = S.cuts;
+                [[maybe_unused]] int marked = S.marked;
                 for (int l = rank; l < lfn * parts; l += C) {
                     const DNode &lf = S.leaf[lf0 + l / parts];
                     if constexpr (F)
@@ -2299,7 +2317,7 @@ __global__ void __launch_bounds__(T) k_direct(const DirectArgs A)
                 {
                     float held;
                     leaves_within<T, F>(S.leaf + lf0, lfn, 1e30f, gain, xr, yr, held);
-                    if (F && (over == 2 || (over && (++cuts_more > F_CUTS || (lfn == 1 && S.leaf[lf0].b - S.leaf[lf0].a == 1)))))
+                    if (F && (over == 2 || (over && (++cuts_made > F_CUTS || (lfn == 1 && S.leaf[lf0].b - S.leaf[lf0].a == 1)))))
                         err = 1;   // more slopes or candidates than the sweep is worth
                     if (over == 1 && lfn == 1) gain = fminf(64.0f, 4.0f * gain);
                     else if (8.0f * (float)nn < held) gain = fmaxf(1.0f / 4096, 0.25f * gain);
@@ -2309,9 +2327,9 @@ __global__ void __launch_bounds__(T) k_direct(const DirectArgs A)
                         // the first leaf with too many candidates: duplicates are marked, the leaves listed again
                         for (int k = rank * T + threadIdx.x; k < (n + 31) / 32; k += T * C) m.dup[k] = 0u;
                         team_sync();
-                        mark_duplicates<T>(pts, n, reinterpret_cast<unsigned *>(wk), slots, rounds, (int)rank, (int)C,
-                                           m.dup, &st->bad);
-                        marked = true;
+                        mark_duplicates<T>(pts, n, reinterpret_cast<unsigned *>(wk), table_slots(), table_rounds(table_slots()),
+                                           (int)rank, (int)C, m.dup, &st->bad);
+                        marked = 1;
                     }
                 }
                 if (rank == 0 && !over) {
@@ -2435,9 +2453,16 @@ __global__ void __launch_bounds__(T) k_direct(const DirectArgs A)
                     flush = false;
                     P = -1;   // minus the intervals for the tree
                 }
+                if (threadIdx.x == 0) {
+                    S.gain = gain;
+                    S.lcap = lcap;
+                    S.regrown = regrown;
+                    S.cuts = cuts_made;
+                    S.marked = marked;
+                }
                 team_sync();
                 if (over && P == 0) {
-                    if (phase > phases) err = 1;
+                    if (phase > phases()) err = 1;
                     mode = err ? M_DONE : M_PAIRS;
                     continue;
                 }
@@ -2495,6 +2520,7 @@ __global__ void __launch_bounds__(T) k_direct(const DirectArgs A)
                 }
                 team_sync();
                 // the best of them that is a pair's slope (fractions need not be)
+                const int slots = table_slots(), rounds = table_rounds(slots);
                 for (int tries = 0; tries < nx; ++tries) {
                     Cand c = cand_empty();
                     for (int k = threadIdx.x; k < nx; k += T) {
@@ -2536,7 +2562,7 @@ __global__ void __launch_bounds__(T) k_direct(const DirectArgs A)
             // ---------------------------------------------------- the next phase
             const bool was_tree = mode == M_TREE;
             if (!F && nx > 0) scored += nx;
-            if (err || phase > phases || (brief && scored > SMALL_SCORES)) {
+            if (err || phase > phases() || (brief() && scored > SMALL_SCORES)) {
                 err = 1;
                 mode = M_DONE;
             } else if (nx > 0) {
@@ -2560,8 +2586,8 @@ __global__ void __launch_bounds__(T) k_direct(const DirectArgs A)
                 }
                 // as many of the leaves as the list is expected to hold
                 float held;
-                lfn = leaves_within<T, F>(S.leaf + lf0, min(nleaf - lf0, lcap), LIST_HOPE * (float)sh.HC, gain, xr, yr,
-                                          held);
+                lfn = leaves_within<T, F>(S.leaf + lf0, min(nleaf - lf0, S.lcap), LIST_HOPE * (float)sh.HC, S.gain,
+                                          xr, yr, held);
                 flush = true;
             } else if (was_tree && P > 0) {
                 mode = M_TREE;
@@ -2607,8 +2633,8 @@ __global__ void __launch_bounds__(T) k_direct(const DirectArgs A)
         } else {
             if (rank == 0 && threadIdx.x == 0) {
                 const int bad = err | __ldcg(&st->bad);
-                if (brief) A.set_done[set] = !bad;
-                if (!(brief && bad)) write_result(A.out + set, best, algo, bad);
+                if (brief()) A.set_done[set] = !bad;
+                if (!(brief() && bad)) write_result(A.out + set, best, algo, bad);
             }
         }
         team_sync();
