@@ -1026,16 +1026,16 @@ __device__ __forceinline__ int leaves_within(const DNode *leaf, int count, float
     return count;
 }
 
-// First position of share `part` of the held points in ord, which lie cell by
-// cell (end[q]: where cell q ends): whole cells.  CTAs that share a leaf sort
-// the points into cells each for itself, and the order inside a cell differs
-// between them, so a cell cut between two of them would lose pairs.
+// The first cell start at or after position p of the held points in ord, which
+// lie cell by cell (end[q]: where cell q ends).  CTAs that share a leaf take
+// blocks of positions by turns (dense cells lie side by side), and the blocks
+// start and end there: every CTA sorts the points into cells for itself, the
+// order inside a cell differs between them, and a cell cut between two of them
+// would lose pairs.
 template <class CELL>
-__device__ __forceinline__ int share_start(int part, int parts, int held, const unsigned *end, const unsigned short *ord,
-                                           CELL cell_of)
+__device__ __forceinline__ int block_start(int p, int held, const unsigned *end, const unsigned short *ord, CELL cell_of)
 {
-    const int p = (int)((long long)held * part / parts);
-    return p == 0 ? 0 : (int)end[cell_of(ord[p - 1])];
+    return p <= 0 ? 0 : p >= held ? held : (int)end[cell_of(ord[p - 1])];
 }
 
 // Shared bytes of list_pairs for NC cells and n points.
@@ -1144,50 +1144,53 @@ __device__ __noinline__ bool list_pairs(const int *pts, int n, const unsigned *d
         constexpr int L = T >= 32 ? 32 : 1;
         const int lane = threadIdx.x % L;
         auto cell_of = [&](int k) { return cell(pts[k]); };
-        const int first = share_start(part, parts, held, cnt, ord, cell_of);
-        const int last = share_start(part + 1, parts, held, cnt, ord, cell_of);
-        for (int e0 = first + threadIdx.x - lane; e0 < last; e0 += T) {
-            const int e = e0 + lane;
-            int pa = 0, n1 = 0, nn = 0, beg2 = 0;
-            if (e < last) {
-                pa = pts[ord[e]];
-                const int q = cell(pa), q2 = (q + 1) & (NC - 1);
-                beg2 = q2 ? (int)cnt[q2 - 1] : 0;
-                n1 = (int)cnt[q] - e - 1;
-                nn = n1 + (int)cnt[q2] - beg2;
-            }
-            int pre = nn;   // inclusive prefix over the warp
-            if constexpr (L == 32) {
-#pragma unroll
-                for (int d = 1; d < 32; d <<= 1) {
-                    const int o = __shfl_up_sync(FULL, pre, d);
-                    if (lane >= d) pre += o;
+        constexpr int BLOCK = T >= 32 ? T : 16;
+        for (int blk = part * BLOCK; blk < held; blk += parts * BLOCK) {
+            const int first = block_start(blk, held, cnt, ord, cell_of);
+            const int last = block_start(blk + BLOCK, held, cnt, ord, cell_of);
+            for (int e0 = first + threadIdx.x - lane; e0 < last; e0 += T) {
+                const int e = e0 + lane;
+                int pa = 0, n1 = 0, nn = 0, beg2 = 0;
+                if (e < last) {
+                    pa = pts[ord[e]];
+                    const int q = cell(pa), q2 = (q + 1) & (NC - 1);
+                    beg2 = q2 ? (int)cnt[q2 - 1] : 0;
+                    n1 = (int)cnt[q] - e - 1;
+                    nn = n1 + (int)cnt[q2] - beg2;
                 }
-            }
-            const int total = L == 32 ? __shfl_sync(FULL, pre, 31) : pre;
-            LMS_DIRECT_COUNT(M_DONE, total);
-            for (int c0 = 0; c0 < total; c0 += L) {
-                const int c = c0 + lane;
-                int src = 0;   // the lane whose candidates hold c
+                int pre = nn;   // inclusive prefix over the warp
                 if constexpr (L == 32) {
 #pragma unroll
-                    for (int d = 16; d >= 1; d >>= 1) {
-                        const int v = __shfl_sync(FULL, pre, src + d - 1);
-                        if (v <= c) src += d;
+                    for (int d = 1; d < 32; d <<= 1) {
+                        const int o = __shfl_up_sync(FULL, pre, d);
+                        if (lane >= d) pre += o;
                     }
-                    src = min(src, 31);
                 }
-                const int u = c - (__shfl_sync(FULL, pre, src) - __shfl_sync(FULL, nn, src));
-                const int k1 = __shfl_sync(FULL, n1, src), k2 = __shfl_sync(FULL, beg2, src);
-                const int p = __shfl_sync(FULL, pa, src);
-                if (c >= total) continue;
-                const int b = ord[u < k1 ? e0 + src + 1 + u : k2 + u - k1];
-                int dy, dx;
-                if (!pair_slope(p, pts[b], dy, dx)) continue;
-                const long long t = (long long)dy << 32;
-                if (!steep && (A * dx > t || B * dx <= t)) continue;
-                const long long k = slope_key(dy, dx);
-                if (k >= A && k < B) table_put(tab, k, dx);
+                const int total = L == 32 ? __shfl_sync(FULL, pre, 31) : pre;
+                LMS_DIRECT_COUNT(M_DONE, total);
+                for (int c0 = 0; c0 < total; c0 += L) {
+                    const int c = c0 + lane;
+                    int src = 0;   // the lane whose candidates hold c
+                    if constexpr (L == 32) {
+#pragma unroll
+                        for (int d = 16; d >= 1; d >>= 1) {
+                            const int v = __shfl_sync(FULL, pre, src + d - 1);
+                            if (v <= c) src += d;
+                        }
+                        src = min(src, 31);
+                    }
+                    const int u = c - (__shfl_sync(FULL, pre, src) - __shfl_sync(FULL, nn, src));
+                    const int k1 = __shfl_sync(FULL, n1, src), k2 = __shfl_sync(FULL, beg2, src);
+                    const int p = __shfl_sync(FULL, pa, src);
+                    if (c >= total) continue;
+                    const int b = ord[u < k1 ? e0 + src + 1 + u : k2 + u - k1];
+                    int dy, dx;
+                    if (!pair_slope(p, pts[b], dy, dx)) continue;
+                    const long long t = (long long)dy << 32;
+                    if (!steep && (A * dx > t || B * dx <= t)) continue;
+                    const long long k = slope_key(dy, dx);
+                    if (k >= A && k < B) table_put(tab, k, dx);
+                }
             }
         }
     }
@@ -1279,32 +1282,35 @@ __device__ __noinline__ void list_pairs_f32(const int2 *pts, int n, long long A,
     const long long err = (1LL << F_YS) + ka + 4;
     constexpr int L = T >= 32 ? 8 : 1;
     auto cell_of = [&](int k) { return cell(pts[k]); };
-    const int first = share_start(part, parts, n, cnt, ord, cell_of);
-    const int last = share_start(part + 1, parts, n, cnt, ord, cell_of);
-    for (int e = first + (int)threadIdx.x / L; e < last; e += T / L) {
-        const int a = ord[e];
-        const int2 pa = pts[a];
-        const int q = cell(pa), q2 = (q + 1) & (NC - 1);
-        const int beg2 = q2 ? (int)cnt[q2 - 1] : 0;
-        const int n1 = (int)cnt[q] - e - 1, nn = n1 + (int)cnt[q2] - beg2;
-        LMS_DIRECT_COUNT(M_DONE, nn);
-        if (*reinterpret_cast<volatile int *>(tab.count) > TABLE * 3 / 4) break;   // the leaf is cut instead
-        for (int u = threadIdx.x % L; u < nn; u += L) {
-            const int b = ord[u < n1 ? e + 1 + u : beg2 + u - n1];
-            const int2 pb = pts[b];
-            // on the grid first: 0 <= dz < dx (B - A), widened
-            long long dx = (long long)pb.x - pa.x, dz = z_at(pb, A, F_YS) - z_at(pa, A, F_YS);
-            if (dx < 0) { dx = -dx; dz = -dz; }
-            if (dz < -err || (double)dz > (double)(dx + 1) * (double)(B - A) + (double)err) continue;
-            double s;
-            if (!slope_f32(f, a, b, s)) continue;
-            const double k = s * f.ratio * (double)(1LL << F_YS);
-            if (!(k >= (double)A && k < (double)B)) continue;
-            if (want) {
-                const unsigned ij = (unsigned)min(a, b) << 16 | (unsigned)max(a, b);
-                if (order_of(s) == *want && *reinterpret_cast<volatile unsigned *>(pair) > ij) atomicMin(pair, ij);
-            } else {
-                table_put(tab, order_of(s), 0);
+    constexpr int BLOCK = T >= 32 ? T / L : 16;
+    for (int blk = part * BLOCK; blk < n; blk += parts * BLOCK) {
+        const int first = block_start(blk, n, cnt, ord, cell_of);
+        const int last = block_start(blk + BLOCK, n, cnt, ord, cell_of);
+        for (int e = first + (int)threadIdx.x / L; e < last; e += T / L) {
+            const int a = ord[e];
+            const int2 pa = pts[a];
+            const int q = cell(pa), q2 = (q + 1) & (NC - 1);
+            const int beg2 = q2 ? (int)cnt[q2 - 1] : 0;
+            const int n1 = (int)cnt[q] - e - 1, nn = n1 + (int)cnt[q2] - beg2;
+            LMS_DIRECT_COUNT(M_DONE, nn);
+            if (*reinterpret_cast<volatile int *>(tab.count) > TABLE * 3 / 4) break;   // the leaf is cut instead
+            for (int u = threadIdx.x % L; u < nn; u += L) {
+                const int b = ord[u < n1 ? e + 1 + u : beg2 + u - n1];
+                const int2 pb = pts[b];
+                // on the grid first: 0 <= dz < dx (B - A), widened
+                long long dx = (long long)pb.x - pa.x, dz = z_at(pb, A, F_YS) - z_at(pa, A, F_YS);
+                if (dx < 0) { dx = -dx; dz = -dz; }
+                if (dz < -err || (double)dz > (double)(dx + 1) * (double)(B - A) + (double)err) continue;
+                double s;
+                if (!slope_f32(f, a, b, s)) continue;
+                const double k = s * f.ratio * (double)(1LL << F_YS);
+                if (!(k >= (double)A && k < (double)B)) continue;
+                if (want) {
+                    const unsigned ij = (unsigned)min(a, b) << 16 | (unsigned)max(a, b);
+                    if (order_of(s) == *want && *reinterpret_cast<volatile unsigned *>(pair) > ij) atomicMin(pair, ij);
+                } else {
+                    table_put(tab, order_of(s), 0);
+                }
             }
         }
     }
