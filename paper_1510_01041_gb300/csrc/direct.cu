@@ -81,8 +81,8 @@ Single float_single_of(int n)
 
 // Float sets: up to 4096 points.  The grid's error (a few 2^-30 of the axes)
 // keeps every slope alive whose width is within about 1e-5 of the optimum:
-// tens of slopes up to here (0.49 ms against 1.29 at n = 2048, 0.64 - 1.0
-// against 2.5 - 2.9 at 4096), thousands above (n = 8192: 1.7 - 9.7 ms against
+// tens of slopes up to here (0.42 - 0.86 ms against 1.24 at n = 2048, 0.75
+// against 2.48 at 4096), thousands above (n = 8192: 1.7 - 9.7 ms against
 // 9.2 - 10.3), each scored by a sort.
 bool direct_f32_ok(int n, int h) { return n >= 16 && n <= 4096 && (long long)h * 4 >= n; }
 
