@@ -1258,17 +1258,21 @@ __device__ __noinline__ void list_pairs_f32(const int2 *pts, int n, long long A,
     __syncthreads();
     const int per = NC / T;
     unsigned sum = 0;
+    constexpr int L = T >= 32 ? 8 : 1, BLOCK = T >= 32 ? T / L : 16, HEAVY = 4 * BLOCK;
     float cand = 0.0f;
+    int heavy = 0;
     for (int r = 0; r < per; ++r) {
         const unsigned c = cnt[threadIdx.x * per + r], c2 = cnt[(threadIdx.x * per + r + 1) & (NC - 1)];
         sum += c;
         cand += (float)c * (0.5f * (float)c + (float)c2);
+        heavy |= c > (unsigned)HEAVY;
     }
     if (candidates_above<T>(cand, F_DENSE, s_warp) && !want) {
         if (threadIdx.x == 0) atomicMax(over, 2);
         __syncthreads();
         return;
     }
+    heavy = __syncthreads_or(heavy);
     int total;
     unsigned run = (unsigned)cta_scan_ex<T>((int)sum, s_warp, total);
     for (int r = 0; r < per; ++r) {
@@ -1280,9 +1284,25 @@ __device__ __noinline__ void list_pairs_f32(const int2 *pts, int n, long long A,
     for (int k = threadIdx.x; k < n; k += T) ord[atomicAdd(&cnt[cell(pts[k])], 1u)] = (unsigned short)k;
     __syncthreads();
     const long long err = (1LL << F_YS) + ka + 4;
-    constexpr int L = T >= 32 ? 8 : 1;
     auto cell_of = [&](int k) { return cell(pts[k]); };
-    constexpr int BLOCK = T >= 32 ? T / L : 16;
+    auto full = [&]() { return *reinterpret_cast<volatile int *>(tab.count) > TABLE * 3 / 4; };   // the leaf is cut instead
+    auto test = [&](int a, int2 pa, int b) {
+        const int2 pb = pts[b];
+        // on the grid first: 0 <= dz < dx (B - A), widened
+        long long dx = (long long)pb.x - pa.x, dz = z_at(pb, A, F_YS) - z_at(pa, A, F_YS);
+        if (dx < 0) { dx = -dx; dz = -dz; }
+        if (dz < -err || (double)dz > (double)(dx + 1) * (double)(B - A) + (double)err) return;
+        double s;
+        if (!slope_f32(f, a, b, s)) return;
+        const double k = s * f.ratio * (double)(1LL << F_YS);
+        if (!(k >= (double)A && k < (double)B)) return;
+        if (want) {
+            const unsigned ij = (unsigned)min(a, b) << 16 | (unsigned)max(a, b);
+            if (order_of(s) == *want && *reinterpret_cast<volatile unsigned *>(pair) > ij) atomicMin(pair, ij);
+        } else {
+            table_put(tab, order_of(s), 0);
+        }
+    };
     for (int blk = part * BLOCK; blk < n; blk += parts * BLOCK) {
         const int first = block_start(blk, n, cnt, ord, cell_of);
         const int last = block_start(blk + BLOCK, n, cnt, ord, cell_of);
@@ -1290,26 +1310,28 @@ __device__ __noinline__ void list_pairs_f32(const int2 *pts, int n, long long A,
             const int a = ord[e];
             const int2 pa = pts[a];
             const int q = cell(pa), q2 = (q + 1) & (NC - 1);
+            if ((int)cnt[q] - (q ? (int)cnt[q - 1] : 0) > HEAVY) continue;
             const int beg2 = q2 ? (int)cnt[q2 - 1] : 0;
             const int n1 = (int)cnt[q] - e - 1, nn = n1 + (int)cnt[q2] - beg2;
             LMS_DIRECT_COUNT(M_DONE, nn);
-            if (*reinterpret_cast<volatile int *>(tab.count) > TABLE * 3 / 4) break;   // the leaf is cut instead
-            for (int u = threadIdx.x % L; u < nn; u += L) {
-                const int b = ord[u < n1 ? e + 1 + u : beg2 + u - n1];
-                const int2 pb = pts[b];
-                // on the grid first: 0 <= dz < dx (B - A), widened
-                long long dx = (long long)pb.x - pa.x, dz = z_at(pb, A, F_YS) - z_at(pa, A, F_YS);
-                if (dx < 0) { dx = -dx; dz = -dz; }
-                if (dz < -err || (double)dz > (double)(dx + 1) * (double)(B - A) + (double)err) continue;
-                double s;
-                if (!slope_f32(f, a, b, s)) continue;
-                const double k = s * f.ratio * (double)(1LL << F_YS);
-                if (!(k >= (double)A && k < (double)B)) continue;
-                if (want) {
-                    const unsigned ij = (unsigned)min(a, b) << 16 | (unsigned)max(a, b);
-                    if (order_of(s) == *want && *reinterpret_cast<volatile unsigned *>(pair) > ij) atomicMin(pair, ij);
-                } else {
-                    table_put(tab, order_of(s), 0);
+            if (full()) break;
+            for (int u = threadIdx.x % L; u < nn; u += L) test(a, pa, ord[u < n1 ? e + 1 + u : beg2 + u - n1]);
+        }
+    }
+    if (heavy) {
+        // cells of many points (points on one line) are shared too, by the points'
+        // indices, which every CTA agrees on: each meets the later ones of its cell
+        for (int blk = part * BLOCK; blk < n; blk += parts * BLOCK) {
+            for (int a = blk + (int)threadIdx.x / L; a < min(n, blk + BLOCK); a += T / L) {
+                const int2 pa = pts[a];
+                const int q = cell(pa), q2 = (q + 1) & (NC - 1);
+                const int beg1 = q ? (int)cnt[q - 1] : 0, n1 = (int)cnt[q] - beg1;
+                if (n1 <= HEAVY) continue;
+                const int beg2 = q2 ? (int)cnt[q2 - 1] : 0, nn = n1 + (int)cnt[q2] - beg2;
+                if (full()) break;
+                for (int u = threadIdx.x % L; u < nn; u += L) {
+                    const int b = ord[u < n1 ? beg1 + u : beg2 + u - n1];
+                    if (u >= n1 || b > a) test(a, pa, b);
                 }
             }
         }

@@ -160,9 +160,10 @@ class Direct:
         return set(out[:n].tolist())
 
     def listed_f32(self, x, y, lo, hi, parts, seed=0):
-        """The same for float points and scaled slope keys: the slopes, as doubles."""
+        """The same for float points and scaled slope keys: the slopes, as doubles.  Seed None: one order (cells of many
+        points are shared by the points' indices, which are the same in every CTA)."""
         rng = np.random.default_rng(seed)
-        order = [rng.permutation(x.size) for _ in range(parts)]
+        order = [np.arange(x.size) if seed is None else rng.permutation(x.size) for _ in range(parts)]
         xy = np.concatenate([np.concatenate([np.float32(x[o]), np.float32(y[o])]) for o in order])
         out = np.zeros(1 << 20, np.int64)
         n = self.lib.host_list_f32(ctypes.c_void_p(xy.ctypes.data), x.size, ctypes.c_int64(lo), ctypes.c_int64(hi), parts,

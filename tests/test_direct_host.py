@@ -44,15 +44,20 @@ def test_shared_leaf_loses_no_slope(D, parts):
         want = set(keys[(keys >= lo) & (keys < hi)].tolist())
         for seed in range(4):
             assert D.listed_i16(x, y, lo, hi, parts, seed) == want, (n, seed)
-        # float points: the frame scales both axes by powers of two
-        xf, yf = np.float32(x + rng.random(n)), np.float32(y + rng.random(n))
-        s = np.subtract(yf[j], yf[i], dtype=np.float64) / np.subtract(xf[j], xf[i], dtype=np.float64)
-        ex, ey = (np.frexp(np.float64(v.max()) - np.float64(v.min()))[1] for v in (xf, yf))
-        k = s * 2.0 ** (int(ex) - int(ey)) * 2.0 ** 29
-        lo, hi = np.floor(np.sort(k)[[k.size // 2, k.size // 2 + 300]]).astype(np.int64).tolist()
-        wantf = set(s[(k >= lo) & (k < hi)].tolist())
-        for seed in range(4):
-            assert D.listed_f32(xf, yf, lo, hi, parts, seed) == wantf, (n, seed)
+        # float points (the frame scales both axes by powers of two); then half of them on one line, in one cell
+        for line in (False, True):
+            xf, yf = np.float32(x + rng.random(n)), np.float32(y + rng.random(n))
+            if line:
+                yf[: n // 2] = np.float32(-0.75) * xf[: n // 2]
+            s = np.subtract(yf[j], yf[i], dtype=np.float64) / np.subtract(xf[j], xf[i], dtype=np.float64)
+            ex, ey = (np.frexp(np.float64(v.max()) - np.float64(v.min()))[1] for v in (xf, yf))
+            scale = 2.0 ** (int(ex) - int(ey) + 29)
+            ks = np.unique(s * scale)
+            at = max(0, int(np.searchsorted(ks, -0.75 * scale)) - 100) if line else ks.size // 2
+            lo, hi = np.floor(ks[[at, min(at + 300, ks.size - 1)]]).astype(np.int64).tolist()
+            want = set(s[(s * scale >= lo) & (s * scale < hi)].tolist())
+            for seed in (None,) if line else range(4):
+                assert D.listed_f32(xf, yf, lo, hi, parts, seed) == want, (n, line, seed)
 
 
 # The counters of ordinary sets at these sizes: at most 16 phases, 32 candidates a point and leaf, 10 slopes scored.
